@@ -18,17 +18,6 @@
 #ifndef VPGS_PIX
 #define VPGS_PIX 2
 #endif
-//   VPGS_BWD_ACC how the backward combines per-warp sums of a Gaussian's 2D
-//                gradient: 0 = one global atomic per warp, 1 = per-warp shared
-//                slots summed per batch, 2 = shared-memory atomics per batch,
-//                -1 = by the tile's warps (1 from 2 warps per tile up, 0 for a
-//                one-warp tile, which has no warps' sums to combine).  0 by
-//                default: with batches of 256 records (render_comp.cu,
-//                VPGS_BWD_BATCH) the shared slots of 1 and 2 would cost resident
-//                blocks
-#ifndef VPGS_BWD_ACC
-#define VPGS_BWD_ACC 0
-#endif
 //   VPGS_DEPTH_SORT_GRID, VPGS_OFFSET_SCAN_GRID  blocks per SM of the depth
 //                sort's passes and of the instance-offset scan (0: what is
 //                resident).  Their item count, the visible pairs, is usually far
@@ -253,6 +242,39 @@ VPGS_D float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+
+VPGS_D float rcp_approx(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Two FP32 values in one register pair and the packed instructions on them
+// (sm_100 and later): each half is rounded to nearest as by the scalar
+// instruction, in one issue slot instead of two.
+typedef unsigned long long f2;
+VPGS_D f2 pack2(float lo, float hi) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+VPGS_D float lo2(f2 v) { return __uint_as_float((uint32_t)v); }
+VPGS_D float hi2(f2 v) { return __uint_as_float((uint32_t)(v >> 32)); }
+VPGS_D f2 add2(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+VPGS_D f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+VPGS_D f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
 }
 
 // alpha of a near-degenerate record at pixel (px, py): d = (px - ux - rx, py - uy - ry) in

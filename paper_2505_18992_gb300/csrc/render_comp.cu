@@ -20,10 +20,12 @@
 // giving dC/dalpha_i = T_i (c_i - B_i), dA/dalpha_i = T_final / (1 - alpha_i).
 // Only g . B enters dL/dalpha (g the pixel's upstream gradient), so each pixel
 // carries that scalar instead of B.
-// Per-Gaussian 2D gradient sums of a warp (in the Gaussian's whitened frame
-// t = W d: sum dpow t1, sum dpow t2, sum dpow t1^2, sum dpow t1 t2, sum dpow
-// t2^2; then opacity, rgb, z) are summed by a transpose reduction (12 shuffles
-// for 10 values) and added with one atomic per value per warp.
+// Per-Gaussian 2D gradient sums of a warp are taken in the Gaussian's whitened frame
+// t = W d: sum dpow t1, sum dpow t2, sum dpow t1^2, sum dpow t1 t2, sum dpow t2^2;
+// then opacity, rgb, z.  Two kernels: the full backward collects its pixels' terms in
+// shared memory and sums them one entry per lane (composite_bwd_kernel); pose
+// tracking sums six of the ten by shuffles (composite_geo_kernel).  Each adds its
+// sums with one atomic per value and warp.
 // Near-degenerate records (negative y half extent) take the double-float pair
 // evaluation (eval_pair_fine): one warp-uniform branch per list entry.
 #include <type_traits>
@@ -48,17 +50,13 @@ VPGS_D TileCoord tile_coord(int t, const CamParams &cam) {
 
 // Each thread owns kPix pixels of its tile column: rows kPix*ly .. kPix*ly + kPix - 1.
 constexpr int kPix = VPGS_PIX;
-#ifndef VPGS_BWD_DIRECT
-#define VPGS_BWD_DIRECT 2
-#endif
-constexpr int kDirect = VPGS_BWD_DIRECT;  // at most this many active lanes: per-lane atomics, no reduction
 constexpr int kMaxThreads = 512;
 #ifndef VPGS_FWD_BATCH
 #define VPGS_FWD_BATCH 2  // records each forward thread stages per batch
 #endif
 constexpr int kFwdBatch = VPGS_FWD_BATCH;
 #ifndef VPGS_BWD_BATCH
-#define VPGS_BWD_BATCH 2  // records each backward thread stages per batch
+#define VPGS_BWD_BATCH 1  // records each thread of the full backward stages per batch (2: 20 KB more, 292 us)
 #endif
 constexpr int kBwdBatch = VPGS_BWD_BATCH;
 // list entries whose alphas the forward evaluates before blending them
@@ -130,6 +128,33 @@ VPGS_D int warp_list(const float4 *s0, const float4 *s1, int n, float2 band, uin
         const uint32_t m = __ballot_sync(0xffffffffu, touch);
         any |= __any_sync(0xffffffffu, f);
         if (touch) list[cnt + __popc(m & below)] = (uint16_t)k;
+        cnt += __popc(m);
+    }
+    __syncwarp();
+    fine = any;
+    return cnt;
+}
+
+// The same list for the backward's packed walk: the byte offsets of the staged
+// records (kBwdRec float4 each), last record first.
+constexpr int kBwdRec = 5;  // float4 per staged record: an odd number keeps 16-byte reads by lane conflict-free
+VPGS_D int warp_list_back(const float4 *s_rec, int n, float2 band, uint16_t *list, int lane, bool &fine, float xmax,
+                          float lg_amin) {
+    const uint32_t below = (1u << lane) - 1u;
+    int cnt = 0;
+    bool any = false;
+    for (int c0 = n - 1; c0 >= 0; c0 -= 32) {
+        const int k = c0 - lane;
+        bool touch = false, f = false;
+        if (k >= 0) {
+            const float4 a = s_rec[kBwdRec * k], b = s_rec[kBwdRec * k + 1];
+            touch = fabsf(a.y - band.x) <= fabsf(b.w) + band.y;
+            f = touch && b.w < 0.f;
+            if (touch && !f) touch = reaches_box(a, b, 0.5f, xmax, band.x - band.y, band.x + band.y, lg_amin);
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, touch);
+        any |= __any_sync(0xffffffffu, f);
+        if (touch) list[cnt + __popc(m & below)] = (uint16_t)(k * (kBwdRec * 16));
         cnt += __popc(m);
     }
     __syncwarp();
@@ -501,28 +526,37 @@ VPGS_D bool pair_grad(PixState &p, int jj, const PairEval &e, const float4 &b, c
     return true;
 }
 
-constexpr int kPartStride = 11;  // floats per (warp, Gaussian) partial, padded against bank conflicts
-
-// register cap of the backward (0: only the 512-thread launch bound).  72
-// registers keep 7 blocks of 4 warps (28 warps) resident per SM: registers are
-// granted in units of 8 per thread, so 73-80 would leave room for 6 blocks.
-// The backward needs no spill under this cap.
-#ifndef VPGS_BWD_MAXREG
-#define VPGS_BWD_MAXREG 72
+// ---------------------------------------------------------------------------
+// Geometric backward (pose tracking: no opacity or colour gradient is asked): the
+// six sums that the means, covariances, depths and the pose need.  One lane per
+// column pair of pixels, branching pair code and a six-value shuffle reduction per
+// entry.  The two-phase form of the full backward took 250 us instead of 345 us here
+// (1M-Gaussian room, 1200x680), but it adds a warp's terms in another order, and a
+// tracking run feeds on its own roundings: the signs of the L1 loss near its minimum
+// amplify them to pose differences beyond those between two runs of this form.
+// ---------------------------------------------------------------------------
+#ifndef VPGS_GEO_BATCH
+#define VPGS_GEO_BATCH 2  // records each thread stages per batch
 #endif
-#if VPGS_BWD_MAXREG > 0
-#define VPGS_BWD_BOUNDS __maxnreg__(VPGS_BWD_MAXREG)
+constexpr int kGeoBatch = VPGS_GEO_BATCH;
+#ifndef VPGS_BWD_DIRECT
+#define VPGS_BWD_DIRECT 2
+#endif
+constexpr int kDirect = VPGS_BWD_DIRECT;  // at most this many active lanes: per-lane atomics, no reduction
+// register cap (0: only the 512-thread launch bound).  72 registers keep 7 blocks of
+// 4 warps resident per SM: registers are granted in units of 8 per thread, so 73-80
+// would leave room for 6 blocks.  The kernel needs no spill under this cap.
+#ifndef VPGS_GEO_MAXREG
+#define VPGS_GEO_MAXREG 72
+#endif
+#if VPGS_GEO_MAXREG > 0
+#define VPGS_GEO_BOUNDS __maxnreg__(VPGS_GEO_MAXREG)
 #else
-#define VPGS_BWD_BOUNDS __launch_bounds__(kMaxThreads)
+#define VPGS_GEO_BOUNDS __launch_bounds__(kMaxThreads)
 #endif
 
-// ACC: how the warps' sums of a Gaussian are combined (VPGS_BWD_ACC): 0 = one
-// global atomic per (warp, Gaussian, slot); 1 = each warp stores its sums in its
-// own shared slots and one thread per Gaussian adds the warps' slots into one
-// global atomic per batch; 2 = shared-memory atomics per batch
-template <int NV, int ACC>
-__global__ void VPGS_BWD_BOUNDS
-composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ ival,
+__global__ void VPGS_GEO_BOUNDS
+composite_geo_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ ival,
                      const uint2 *__restrict__ ranges, const uint32_t *__restrict__ order, int n_tiles,
                      CamParams cam, OptParams o,
                      const float *__restrict__ t_final, const int32_t *__restrict__ n_iter,
@@ -531,12 +565,10 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                      const uint32_t *status, uint32_t *work) {
     grid_dep_enter();
     extern __shared__ float4 smem[];
-    const int NT = blockDim.x * kBwdBatch;  // records per batch
-    const int NW = blockDim.x >> 5;
+    const int NT = blockDim.x * kGeoBatch;  // records per batch
     float4 *s0 = smem, *s1 = smem + NT, *s2 = smem + 2 * NT;
     uint32_t *s_id = reinterpret_cast<uint32_t *>(smem + 3 * NT);
     uint16_t *s_wl = reinterpret_cast<uint16_t *>(s_id + NT);             // [NW][NT] per-warp lists
-    float *s_part = reinterpret_cast<float *>(s_wl + (size_t)NW * NT);  // [NW][NT][kPartStride]
     __shared__ int s_tile;
     __shared__ int s_max;
     if (*status != 0u) return;
@@ -549,19 +581,9 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
     const float2 band = warp_rows(pyl);
     const float lg_amin = __log2f(o.alpha_min);
     uint16_t *wl = s_wl + (size_t)warp * NT;
-    float *my_part = s_part + (size_t)warp * NT * kPartStride;
+    constexpr int NV = 6;
     const int rs = red_slot<NV>(lane);
     const int slot = rs >= 0 ? g2d_slot<NV>(rs) : -1;
-    // hands one warp total (this lane's slot) of Gaussian k to the combination scheme
-    auto put = [&](int k, float val) {
-        if (ACC == 0) {
-            if (val != 0.f) atomicAdd(g2d + 10 * (int64_t)s_id[k] + slot, val);
-        } else if (ACC == 1) {
-            my_part[k * kPartStride + slot] = val;
-        } else {
-            if (val != 0.f) atomicAdd(s_part + k * kPartStride + slot, val);
-        }
-    };
     int t = blockIdx.x;
     for (;;) {
         if (work) {
@@ -613,7 +635,7 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
             const int nb = b1 - b0;
             __syncthreads();
 #pragma unroll 1
-            for (int u = 0; u < kBwdBatch; ++u) {
+            for (int u = 0; u < kGeoBatch; ++u) {
                 const int k = tid + u * (int)blockDim.x;
                 if (b0 + k < b1) {
                     const uint32_t id = ival[b0 + k];
@@ -621,10 +643,6 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                     s_id[k] = id;
                 }
             }
-            if (ACC == 1)
-                for (int e = lane; e < nb * kPartStride; e += 32) my_part[e] = 0.f;
-            if (ACC == 2)
-                for (int e = tid; e < nb * kPartStride; e += (int)blockDim.x) s_part[e] = 0.f;
             __syncthreads();
             const int k_end = min(nb, warp_max - (b0 - start));  // warp-uniform
             bool any_fine;
@@ -660,7 +678,7 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                 else
                     act = grads(std::false_type{});
                 const uint32_t am = __ballot_sync(0xffffffffu, act);
-                if (ACC == 0 && am != 0u && __popc(am) <= kDirect) {
+                if (am != 0u && __popc(am) <= kDirect) {
                     // few active lanes: their own atomics beat a reduction
                     if (act) {
                         float *dst = g2d + 10 * (int64_t)s_id[kk];
@@ -670,28 +688,338 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                     }
                 } else if (am != 0u) {
                     warp_reduce(v, lane);
-                    if (slot >= 0) put(kk, v[0]);
+                    if (slot >= 0 && v[0] != 0.f) atomicAdd(g2d + 10 * (int64_t)s_id[kk] + slot, v[0]);
                 }
             }
             };
             if (any_fine) walk(std::true_type{});
             else walk(std::false_type{});
-            if (ACC != 0) {
-                __syncthreads();
-                // one thread per Gaussian of the batch: one global atomic per value
-                for (int k = tid; k < nb; k += (int)blockDim.x) {
-                    float *dst = g2d + 10 * (int64_t)s_id[k];
+        }
+        if (!work) return;
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Backward.  The ten 2D gradient sums of a Gaussian are linear in two numbers per
+// pixel, its blend weight w and dpow (the gradient of the exponent):
+//   sum w (g_r, g_g, g_b, g_z)   and   sum dpow (1, t1, t2, t1^2, t1 t2, t2^2)
+// (sum dpow / o is the opacity's).  So a warp works in two phases:
+//   1. one lane per column pair of pixels (two rows), as in the forward: walk the
+//      list back to front, update T and beta, and leave (w, dpow) of both pixels in
+//      a slot of shared memory.  Entries that blend into no pixel take no slot.
+//   2. when kSlots entries are collected (or the batch ends): kSlots x (32 / kSlots)
+//      lanes, each summing one entry over its share of the warp's pixels in
+//      registers, then log2(32 / kSlots) transpose steps and one global atomic per
+//      (warp, Gaussian, slot).
+// Both phases do their arithmetic on the two rows of a column at once with the
+// packed FP32 instructions (fma.rn.f32x2), which round each half as the scalar
+// ones do.  Lanes that do not blend take part with alpha = 0 (T and beta then keep
+// their values exactly), so a step has no branch but the one on the warp's vote.
+// Bound: the shared-memory pipe and latency (issue active 60 %, LSU data pipe 58 %, FMA
+// pipe 42 %; 20 warps per SM).  103 warp instructions per listed entry, against 189 of
+// the branching pair code and ten-value shuffle reduction it replaces.  Measured, old ->
+// new: 1M-Gaussian room 1200x680 393 -> 278 us, 8 keyframes of 2M 1848 -> 1369 us, four
+// full-HD views of 34k visible Gaussians 1111 -> 785 us, 10k Gaussians 320x240 41 -> 24 us.
+// kSlots 16 halves the transpose steps but takes 16 KB more per block: 322 us (room).
+// The shuffle form remains for the batches that hold a near-degenerate record, and for
+// pixels or records whose magnitudes could turn 0 * x into a NaN (kOdd).
+// ---------------------------------------------------------------------------
+#ifndef VPGS_BWD_SLOTS
+#define VPGS_BWD_SLOTS 8
+#endif
+constexpr int kSlots = VPGS_BWD_SLOTS;
+#ifndef VPGS_BWD_UNROLL
+#define VPGS_BWD_UNROLL 2
+#endif
+constexpr int kBwdUnroll = VPGS_BWD_UNROLL;
+static_assert(kSlots == 8 || kSlots == 16, "entries per flush");
+constexpr int kTermStride = 33;           // float4 per slot: 32 lanes, padded against bank conflicts
+constexpr int kPixSize = 64 + 32 / kSlots;  // the lanes' gradients: 2 float4 each, one of padding per part of phase 2
+// |upstream gradient| and |colour, depth| from which a pixel or record takes the
+// branching walk: below it every product of the masked form stays finite
+constexpr float kOdd = 1e15f;
+
+static_assert(kPix == 2, "the packed forms hold two rows per lane");
+
+// register cap (0: only the 512-thread launch bound).  80: 6 blocks of 4 warps per SM, as
+// many as the shared memory allows; 72: 285 us, 96: 285 us (room; 278 at 80)
+#ifndef VPGS_BWD_MAXREG
+#define VPGS_BWD_MAXREG 80
+#endif
+#if VPGS_BWD_MAXREG > 0
+#define VPGS_BWD_BOUNDS __maxnreg__(VPGS_BWD_MAXREG)
+#else
+#define VPGS_BWD_BOUNDS __launch_bounds__(kMaxThreads)
+#endif
+
+__global__ void VPGS_BWD_BOUNDS
+composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ ival,
+                     const uint2 *__restrict__ ranges, const uint32_t *__restrict__ order, int n_tiles,
+                     CamParams cam, OptParams o,
+                     const float *__restrict__ t_final, const int32_t *__restrict__ n_iter,
+                     const float *__restrict__ dL_drgb, const float *__restrict__ dL_ddepth,
+                     const float *__restrict__ dL_dalpha, float *__restrict__ g2d,
+                     const uint32_t *status, uint32_t *work) {
+    grid_dep_enter();
+    constexpr int NV = 10;
+    extern __shared__ float4 smem[];
+    const int NT = blockDim.x * kBwdBatch;  // records per batch
+    const int NW = blockDim.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // records: s0, s1 as in the forward, the colour and depth doubled (r, r, g, g), (b, b, z, z), the id
+    float4 *s_rec = smem;
+    float4 *s_term = smem + kBwdRec * NT + warp * (kSlots * kTermStride);           // this warp's (w, w, dpow, dpow)
+    float4 *s_pix = smem + kBwdRec * NT + NW * (kSlots * kTermStride) + warp * kPixSize;  // this warp's -g
+    uint16_t *wl = reinterpret_cast<uint16_t *>(smem + kBwdRec * NT + NW * (kSlots * kTermStride + kPixSize)) +
+                   (size_t)warp * NT;  // this warp's list
+    auto rec_at = [&](int off) { return reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(s_rec) + off); };
+    __shared__ int s_tile;
+    __shared__ int s_max;
+    __shared__ int s_odd;
+    if (*status != 0u) return;
+    const int lx = tid % cam.tile_w, ly = tid / cam.tile_w;
+    const float pxl = (float)lx + 0.5f;
+    float pyl[kPix];
 #pragma unroll
-                    for (int sl = 0; sl < 10; ++sl) {
-                        float acc = 0.f;
-                        if (ACC == 1) {
-                            for (int w = 0; w < NW; ++w) acc += s_part[((size_t)w * NT + k) * kPartStride + sl];
-                        } else {
-                            acc = s_part[k * kPartStride + sl];
+    for (int q = 0; q < kPix; ++q) pyl[q] = (float)(kPix * ly + q) + 0.5f;
+    const float2 band = warp_rows(pyl);
+    const float lg_amin = __log2f(o.alpha_min);
+    const f2 one2 = pack2(1.f, 1.f);
+    int t = blockIdx.x;
+    for (;;) {
+        if (work) {
+            if (tid == 0) s_tile = (int)atomicAdd(work, 1u);
+            __syncthreads();
+            t = s_tile;
+        }
+        if (tid == 0) {
+            s_max = 0;
+            s_odd = 0;
+        }
+        __syncthreads();
+        if (t >= n_tiles) return;
+        const int tile = order ? (int)order[t] : t;  // launch order -> global tile id
+        const TileCoord tc = tile_coord(tile, cam);
+        const int px = tc.tx * cam.tile_w + lx;
+        const float ox = (float)(tc.tx * cam.tile_w), oy = (float)(tc.ty * cam.tile_h);
+        const float xmax = fminf((float)cam.tile_w, (float)cam.W - ox) - 0.5f;  // last pixel centre column
+        const uint2 rg = ranges[tile];
+        const int start = (int)rg.x;
+        const int64_t HW = (int64_t)cam.H * cam.W;
+        // per pixel: T, the negated upstream gradient ng, -dL/dalpha * T_final (ngat) and
+        // beta = g . B, the upstream gradient dotted with the colour / depth behind the
+        // current Gaussian (B starts at the background)
+        float T[kPix], ng0[kPix], ng1[kPix], ng2[kPix], ngd[kPix], ngat[kPix], beta[kPix];
+        int last[kPix];
+        int my_max = 0;
+        bool odd = false;
+#pragma unroll
+        for (int q = 0; q < kPix; ++q) {
+            T[q] = 1.f;
+            ng0[q] = ng1[q] = ng2[q] = ngd[q] = 0.f;
+            last[q] = 0;
+            float gA = 0.f;
+            const int py = tc.ty * cam.tile_h + kPix * ly + q;
+            if (px < cam.W && py < cam.H) {
+                const int64_t pix = (int64_t)tc.v * HW + (int64_t)py * cam.W + px;
+                T[q] = t_final[pix];
+                last[q] = n_iter[pix];
+                if (dL_drgb) {
+                    const float *gp = dL_drgb + (int64_t)tc.v * 3 * HW + (int64_t)py * cam.W + px;
+                    ng0[q] = -gp[0]; ng1[q] = -gp[HW]; ng2[q] = -gp[2 * HW];
+                }
+                if (dL_ddepth) ngd[q] = -dL_ddepth[pix];
+                if (dL_dalpha) gA = dL_dalpha[pix];
+            }
+            ngat[q] = -(gA * T[q]);  // T holds T_final here
+            beta[q] = -fmaf(ng0[q], o.bg0, fmaf(ng1[q], o.bg1, ng2[q] * o.bg2));
+            odd |= !(fmaxf(fmaxf(fabsf(ng0[q]), fabsf(ng1[q])), fmaxf(fabsf(ng2[q]), fabsf(ngd[q]))) < kOdd) ||
+                   !(fabsf(ngat[q]) < kOdd && fabsf(beta[q]) < kOdd) || ng0[q] != ng0[q] || ng1[q] != ng1[q] ||
+                   ng2[q] != ng2[q] || ngd[q] != ngd[q];
+            my_max = max(my_max, last[q]);
+        }
+        const bool warp_odd = __any_sync(0xffffffffu, odd);
+        s_pix[2 * lane + lane / kSlots] = make_float4(ng0[0], ng0[1], ng1[0], ng1[1]);
+        s_pix[2 * lane + lane / kSlots + 1] = make_float4(ng2[0], ng2[1], ngd[0], ngd[1]);
+        f2 T2 = pack2(T[0], T[1]), beta2 = pack2(beta[0], beta[1]);
+        const f2 ng02 = pack2(ng0[0], ng0[1]), ng12 = pack2(ng1[0], ng1[1]), ng22 = pack2(ng2[0], ng2[1]),
+                 ngd2 = pack2(ngd[0], ngd[1]), ngat2 = pack2(ngat[0], ngat[1]);
+        // the warp's own list length: warps whose pixels stop early skip the tail
+        const int warp_max = (int)__reduce_max_sync(0xffffffffu, (unsigned)my_max);
+        if (lane == 0 && warp_max > 0) atomicMax(&s_max, warp_max);
+        __syncthreads();
+        const int list_end = start + min(s_max, (int)rg.y - start);  // n_iter never exceeds the list
+        for (int b1 = list_end; b1 > start; b1 -= NT) {
+            const int b0 = max(start, b1 - NT);
+            const int nb = b1 - b0;
+            __syncthreads();
+#pragma unroll 1
+            for (int u = 0; u < kBwdBatch; ++u) {
+                const int k = tid + u * (int)blockDim.x;
+                if (b0 + k < b1) {
+                    const uint32_t id = ival[b0 + k];
+                    float4 a, b, c;
+                    stage(rec[id], ox, oy, a, b, c);
+                    float4 *d = s_rec + kBwdRec * k;
+                    d[0] = a;
+                    d[1] = b;
+                    d[2] = make_float4(c.x, c.x, c.y, c.y);
+                    d[3] = make_float4(c.z, c.z, c.w, c.w);
+                    d[4].x = __uint_as_float(id);
+                    if (!(fmaxf(fmaxf(fabsf(c.x), fabsf(c.y)), fmaxf(fabsf(c.z), fabsf(c.w))) < kOdd)) s_odd = 1;
+                }
+            }
+            __syncthreads();
+            const int k_end = min(nb, warp_max - (b0 - start));  // warp-uniform
+            bool any_fine;
+            const int nl = warp_list_back(s_rec, k_end, band, wl, lane, any_fine, xmax, lg_amin);
+            const int base = b0 - start;  // list position of the batch's first record
+            if (any_fine || warp_odd || s_odd != 0) {  // warp-uniform
+                // entry by entry, each in its precision form, the warp's sums by shuffles
+                PixState ps[kPix];
+#pragma unroll
+                for (int q = 0; q < kPix; ++q) {
+                    PixState &p = ps[q];
+                    p.T = q ? hi2(T2) : lo2(T2);
+                    p.beta = q ? hi2(beta2) : lo2(beta2);
+                    p.gAT = -(q ? hi2(ngat2) : lo2(ngat2));
+                    p.gC0 = -(q ? hi2(ng02) : lo2(ng02));
+                    p.gC1 = -(q ? hi2(ng12) : lo2(ng12));
+                    p.gC2 = -(q ? hi2(ng22) : lo2(ng22));
+                    p.gD = -(q ? hi2(ngd2) : lo2(ngd2));
+                    p.last = last[q];
+                }
+                const int slot = red_slot<NV>(lane);
+                for (int i = 0; i < nl; ++i) {
+                    const float4 *r = rec_at(wl[i]);
+                    const int kk = wl[i] / (kBwdRec * 16);
+                    const uint32_t id = __float_as_uint(r[4].x);
+                    const float4 a = r[0], b = r[1], c2 = r[2], c3 = r[3];
+                    const float4 c = make_float4(c2.x, c2.z, c3.x, c3.z);
+                    float v[NV];
+#pragma unroll
+                    for (int q = 0; q < NV; ++q) v[q] = 0.f;
+                    auto grads = [&](auto fine) -> bool {
+                        constexpr bool kFine = decltype(fine)::value;
+                        float4 f;
+                        if constexpr (kFine) f = fine_extra(rec[id], ox, oy, a.x, a.y);
+                        const float2 t0 = kFine ? make_float2(0.f, 0.f) : first_row(pxl, pyl[0], a, b);
+                        bool any = false;
+#pragma unroll
+                        for (int q = 0; q < kPix; ++q) {
+                            const PairEval e = eval_staged<kFine>(q, t0.x, t0.y, pxl, pyl[q], a, b, f, o.alpha_max);
+                            any |= pair_grad(ps[q], base + kk, e, b, c, o, v);
                         }
-                        if (acc != 0.f) atomicAdd(dst + sl, acc);
+                        return any;
+                    };
+                    const bool act = b.w < 0.f ? grads(std::true_type{}) : grads(std::false_type{});
+                    if (__any_sync(0xffffffffu, act)) {
+                        warp_reduce(v, lane);
+                        if (slot >= 0 && v[0] != 0.f) atomicAdd(g2d + 10 * (int64_t)id + slot, v[0]);
                     }
                 }
+                T2 = pack2(ps[0].T, ps[1].T);
+                beta2 = pack2(ps[0].beta, ps[1].beta);
+                continue;
+            }
+            const int l0 = (last[0] - base) * (kBwdRec * 16), l1 = (last[1] - base) * (kBwdRec * 16);
+            for (int g = 0; g < nl; g += kSlots) {
+                const int n = min(kSlots, nl - g);  // warp-uniform
+                // phase 1
+#pragma unroll kBwdUnroll
+                for (int i = 0; i < n; ++i) {
+                    const int off = wl[g + i];
+                    const float4 *r = rec_at(off);
+                    const float4 a = r[0], b = r[1], c2 = r[2], c3 = r[3];
+                    const float2 t0 = first_row(pxl, pyl[0], a, b);
+                    const f2 t12 = pack2(t0.x, t0.x + a.w), t22 = pack2(t0.y, t0.y + b.y);
+                    const f2 q = fma2(t12, t12, mul2(t22, t22));
+                    const float r0 = b.z * ex2_approx(-lo2(q)), r1 = b.z * ex2_approx(-hi2(q));
+                    const float al0 = fminf(o.alpha_max, r0), al1 = fminf(o.alpha_max, r1);
+                    // negated alphas, zero where the pixel does not blend
+                    const f2 na = pack2(al0 >= o.alpha_min && off < l0 ? -al0 : 0.f,
+                                        al1 >= o.alpha_min && off < l1 ? -al1 : 0.f);
+                    const f2 om = add2(one2, na);  // 1 - alpha >= 1 - alpha_max > 0
+                    const f2 iom = pack2(rcp_approx(lo2(om)), rcp_approx(hi2(om)));
+                    T2 = mul2(T2, iom);
+                    // ed = g . (B - c); dL/dalpha_i = T_i g . (c_i - B_i) + dL/dalpha T_final / (1 - alpha_i)
+                    const f2 ed = fma2(ng02, pack2(c2.x, c2.y),
+                                       fma2(ng12, pack2(c2.z, c2.w),
+                                            fma2(ng22, pack2(c3.x, c3.y), fma2(ngd2, pack2(c3.z, c3.w), beta2))));
+                    const f2 ndA = fma2(ed, T2, mul2(ngat2, iom));
+                    beta2 = fma2(na, ed, beta2);  // B <- B + alpha (c - B)
+                    const f2 nw = mul2(na, T2);
+                    const f2 dp = mul2(ndA, na);
+                    // a clamped alpha has zero derivative
+                    s_term[i * kTermStride + lane] = make_float4(lo2(nw), hi2(nw), r0 <= o.alpha_max ? lo2(dp) : 0.f,
+                                                                 r1 <= o.alpha_max ? hi2(dp) : 0.f);
+                }
+                __syncwarp();
+                // phase 2
+                const int e = lane & (kSlots - 1), part = lane / kSlots;
+                constexpr int kShare = kSlots;  // lanes (pixel pairs) of phase 1 per part: 32 / (32 / kSlots)
+                const float4 *r = rec_at(wl[g + (e < n ? e : 0)]);
+                const float4 a = r[0], b = r[1];
+                f2 v[NV];
+#pragma unroll
+                for (int q = 0; q < NV; ++q) v[q] = pack2(0.f, 0.f);
+                const float4 *term = s_term + e * kTermStride + part * kShare;
+                const float4 *pix = s_pix + (2 * kShare + 1) * part;
+#pragma unroll
+                for (int h = 0; h < kShare; h += 4) {
+                    // four lanes in a row of the tile (tile_w is a multiple of 4)
+                    const int j = part * kShare + h;
+                    const float x0 = (float)(j & (cam.tile_w - 1)) + 0.5f;
+                    const float dy = (float)(kPix * ((warp * 32 + j) >> cam.tw_shift)) + 0.5f - a.y;
+                    const float y1 = a.w * dy, y2 = b.y * dy;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float4 tm = term[h + i];
+                        const float dx = (x0 + (float)i) - a.x;
+                        const float t1 = fmaf(a.z, dx, y1), t2 = fmaf(b.x, dx, y2);
+                        const f2 t12 = pack2(t1, t1 + a.w), t22 = pack2(t2, t2 + b.y);
+                        const f2 w = pack2(tm.x, tm.y), p = pack2(tm.z, tm.w);
+                        const f2 pt1 = mul2(p, t12), pt2 = mul2(p, t22);
+                        v[0] = add2(v[0], pt1);
+                        v[1] = add2(v[1], pt2);
+                        v[2] = fma2(pt1, t12, v[2]);
+                        v[3] = fma2(pt1, t22, v[3]);
+                        v[4] = fma2(pt2, t22, v[4]);
+                        const float4 g0 = pix[2 * (h + i)], g1 = pix[2 * (h + i) + 1];
+                        v[5] = add2(v[5], p);
+                        v[6] = fma2(w, pack2(g0.x, g0.y), v[6]);
+                        v[7] = fma2(w, pack2(g0.z, g0.w), v[7]);
+                        v[8] = fma2(w, pack2(g1.x, g1.y), v[8]);
+                        v[9] = fma2(w, pack2(g1.z, g1.w), v[9]);
+                    }
+                }
+                float rs[NV];
+#pragma unroll
+                for (int q = 0; q < NV; ++q) rs[q] = lo2(v[q]) + hi2(v[q]);
+                rs[5] = __fdividef(rs[5], b.z);  // dL/do = sum dpow / o
+                // the parts' sums, the values spread over the lanes that held them
+                constexpr int H = (NV + 1) / 2;
+                half_step<NV, 16>(rs, lane);
+                int lo = (lane & 16) ? H : 0, nq = (lane & 16) ? NV - H : H;
+                if constexpr (kSlots == 8) {
+                    constexpr int Q = (H + 1) / 2;
+                    half_step<H, 8>(rs, lane);
+                    if (lane & 8) {
+                        lo += Q;
+                        nq -= Q;
+                    } else {
+                        nq = min(nq, Q);
+                    }
+                }
+                if (e < n) {
+                    float *dst = g2d + 10 * (int64_t)__float_as_uint(r[4].x);
+                    constexpr int M = kSlots == 8 ? (H + 1) / 2 : H;
+#pragma unroll
+                    for (int q = 0; q < M; ++q)
+                        if (q < nq && rs[q] != 0.f) atomicAdd(dst + lo + q, rs[q]);
+                }
+                __syncwarp();
             }
         }
         if (!work) return;
@@ -700,14 +1028,17 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
 }
 
 // dynamic shared memory of a compositing block of `threads` threads staging
-// `records` per batch: forward s0-s3 and the warps' lists; backward s0-s2, the
-// ids, the lists and the per-Gaussian partial sums of the combination scheme
-static size_t comp_smem(int threads, int records, bool bwd, int acc = 0) {
-    const size_t warps = (size_t)threads / 32;
-    const size_t parts = acc == 1 ? warps * records * kPartStride : (acc == 2 ? (size_t)records * kPartStride : 0);
-    const size_t lists = sizeof(uint16_t) * warps * records;
-    return sizeof(float4) * (bwd ? 3 : 4) * records + lists +
-           (bwd ? sizeof(uint32_t) * records + sizeof(float) * parts : 0);
+// `records` per batch: forward s0-s3 and the warps' lists; geometric backward s0-s2,
+// the ids and the lists; full backward the staged records, the warps' term slots and
+// pixel gradients, and the lists
+static size_t list_bytes(int threads, int records) { return sizeof(uint16_t) * (size_t)(threads / 32) * records; }
+static size_t fwd_smem(int threads, int records) { return sizeof(float4) * 4 * records + list_bytes(threads, records); }
+static size_t geo_smem(int threads, int records) {
+    return (sizeof(float4) * 3 + sizeof(uint32_t)) * records + list_bytes(threads, records);
+}
+static size_t bwd_smem(int threads, int records) {
+    return sizeof(float4) * (kBwdRec * (size_t)records + (size_t)(threads / 32) * (kSlots * kTermStride + kPixSize)) +
+           list_bytes(threads, records);
 }
 
 static int persistent_grid(const void *kernel, int B, size_t smem, int per_sm, int n_tiles) {
@@ -723,7 +1054,7 @@ cudaError_t launch_composite_fwd(const RenderWs &ws, const uint32_t *ival, int V
                                  int persistent_ctas, cudaStream_t s) {
     const int B = cam.tile_w * cam.tile_h / kPix;
     const int n_tiles = V * cam.T;
-    const size_t sm = comp_smem(B, B * kFwdBatch, false);
+    const size_t sm = fwd_smem(B, B * kFwdBatch);
     uint32_t *work = nullptr;
     int grid = n_tiles;
     if (persistent_ctas > 0) {
@@ -733,7 +1064,7 @@ cudaError_t launch_composite_fwd(const RenderWs &ws, const uint32_t *ival, int V
         grid = persistent_grid((const void *)composite_fwd_kernel, B, sm, persistent_ctas, n_tiles);
     }
     if (grid == 0) return cudaSuccess;
-    if (sm > 48 * 1024)
+    if (sm > 40 * 1024)
         cudaFuncSetAttribute((const void *)composite_fwd_kernel,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     VPGS_LAUNCH("composite_fwd", s,
@@ -743,55 +1074,32 @@ cudaError_t launch_composite_fwd(const RenderWs &ws, const uint32_t *ival, int V
     return cudaGetLastError();
 }
 
-template <int NV, int ACC>
-static cudaError_t composite_bwd_as(const RenderWs &ws, const uint32_t *ival, int V, const CamParams &cam,
-                                    const OptParams &o, const vpgs_images &fwd, const float *dL_drgb,
-                                    const float *dL_ddepth, const float *dL_dalpha, int persistent_ctas,
-                                    cudaStream_t s) {
+cudaError_t launch_composite_bwd(const RenderWs &ws, const uint32_t *ival, int V,
+                                 const CamParams &cam, const OptParams &o, const vpgs_images &fwd,
+                                 const float *dL_drgb, const float *dL_ddepth,
+                                 const float *dL_dalpha, bool geometric_only, int persistent_ctas,
+                                 cudaStream_t s) {
     const int B = cam.tile_w * cam.tile_h / kPix;
     const int n_tiles = V * cam.T;
-    const size_t sm = comp_smem(B, B * kBwdBatch, true, ACC);
-    const void *kern = (const void *)composite_bwd_kernel<NV, ACC>;
+    const auto kern = geometric_only ? composite_geo_kernel : composite_bwd_kernel;
+    const size_t sm = geometric_only ? geo_smem(B, B * kGeoBatch) : bwd_smem(B, B * kBwdBatch);
+    // (the kernels' few static words count towards the default limit of 48 KB)
+    if (sm > 40 * 1024)
+        cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     uint32_t *work = nullptr;
     int grid = n_tiles;
     if (persistent_ctas > 0) {
         work = ws.counters + CNT_WORK;
         cudaError_t e = cudaMemsetAsync(work, 0, sizeof(uint32_t), s);
         if (e != cudaSuccess) return e;
-        grid = persistent_grid(kern, B, sm, persistent_ctas, n_tiles);
+        grid = persistent_grid((const void *)kern, B, sm, persistent_ctas, n_tiles);
     }
     if (grid == 0) return cudaSuccess;
-    if (sm > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     VPGS_LAUNCH("composite_bwd", s,
-                launch_k(composite_bwd_kernel<NV, ACC>, grid, B, sm, s, ws.rec, ival, ws.ranges,
+                launch_k(kern, grid, B, sm, s, ws.rec, ival, ws.ranges,
                          VPGS_TILE_ORDER ? (const uint32_t *)ws.tile_order : nullptr, n_tiles, cam, o,
                          fwd.t_final, fwd.n_iter, dL_drgb, dL_ddepth, dL_dalpha, ws.g2d, ws.status, work));
     return cudaGetLastError();
-}
-
-template <int NV>
-static cudaError_t composite_bwd_nv(int acc, const RenderWs &ws, const uint32_t *ival, int V,
-                                    const CamParams &cam, const OptParams &o, const vpgs_images &fwd,
-                                    const float *dL_drgb, const float *dL_ddepth, const float *dL_dalpha,
-                                    int persistent_ctas, cudaStream_t s) {
-    switch (acc) {
-    case 1: return composite_bwd_as<NV, 1>(ws, ival, V, cam, o, fwd, dL_drgb, dL_ddepth, dL_dalpha, persistent_ctas, s);
-    case 2: return composite_bwd_as<NV, 2>(ws, ival, V, cam, o, fwd, dL_drgb, dL_ddepth, dL_dalpha, persistent_ctas, s);
-    default: return composite_bwd_as<NV, 0>(ws, ival, V, cam, o, fwd, dL_drgb, dL_ddepth, dL_dalpha, persistent_ctas, s);
-    }
-}
-
-cudaError_t launch_composite_bwd(const RenderWs &ws, const uint32_t *ival, int V,
-                                 const CamParams &cam, const OptParams &o, const vpgs_images &fwd,
-                                 const float *dL_drgb, const float *dL_ddepth,
-                                 const float *dL_dalpha, bool geometric_only, int persistent_ctas,
-                                 cudaStream_t s) {
-    // per-warp shared slots pay off as soon as a tile has warps' sums to combine
-    const int warps = cam.tile_w * cam.tile_h / kPix / 32;
-    const int acc = VPGS_BWD_ACC >= 0 ? VPGS_BWD_ACC : (warps >= 2 ? 1 : 0);
-    return geometric_only
-               ? composite_bwd_nv<6>(acc, ws, ival, V, cam, o, fwd, dL_drgb, dL_ddepth, dL_dalpha, persistent_ctas, s)
-               : composite_bwd_nv<10>(acc, ws, ival, V, cam, o, fwd, dL_drgb, dL_ddepth, dL_dalpha, persistent_ctas, s);
 }
 
 }  // namespace vpgs
