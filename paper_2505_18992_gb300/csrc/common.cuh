@@ -261,6 +261,7 @@ VPGS_D f2 pack2(float lo, float hi) {
 }
 VPGS_D float lo2(f2 v) { return __uint_as_float((uint32_t)v); }
 VPGS_D float hi2(f2 v) { return __uint_as_float((uint32_t)(v >> 32)); }
+VPGS_D f2 neg2(f2 v) { return pack2(-lo2(v), -hi2(v)); }
 VPGS_D f2 add2(f2 a, f2 b) {
     f2 r;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));

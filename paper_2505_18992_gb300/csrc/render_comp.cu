@@ -1,9 +1,9 @@
 // Front-to-back alpha compositing per tile, and its backward pass.
 //
-// One CTA renders one tile (tile_w x tile_h threads, one pixel each), or, in
-// persistent mode, a fixed number of CTAs per SM pull tiles from a work queue.
-// The tile's depth-ordered Gaussian list is staged through shared memory in
-// batches of one record per thread; each pixel walks the batch in order:
+// One CTA renders one tile (tile_w x tile_h / 2 threads, two rows of a column each),
+// or, in persistent mode, a fixed number of CTAs per SM pull tiles from a work queue.
+// The tile's depth-ordered Gaussian list is staged through shared memory in batches
+// of one or two records per thread; each pixel walks the batch in order:
 //   alpha = min(alpha_max, o 2^-((w1.d)^2 + (w2.d)^2)), d = pixel - mean, with
 //           the whitening rows w scaled by sqrt(log2(e)/2) when the record is made
 //   skip alpha < alpha_min; stop before T (1 - alpha) < t_min
@@ -59,9 +59,9 @@ constexpr int kFwdBatch = VPGS_FWD_BATCH;
 #define VPGS_BWD_BATCH 1  // records each thread of the full backward stages per batch (2: 20 KB more, 292 us)
 #endif
 constexpr int kBwdBatch = VPGS_BWD_BATCH;
-// list entries whose alphas the forward evaluates before blending them
+// list entries whose alphas the forward evaluates before blending them (see VPGS_FWD_MAXREG)
 #ifndef VPGS_FWD_WALK
-#define VPGS_FWD_WALK 2
+#define VPGS_FWD_WALK 8
 #endif
 constexpr int kWalk = VPGS_FWD_WALK;
 
@@ -102,14 +102,10 @@ VPGS_D bool reaches_box(const float4 &a, const float4 &b, float x0, float x1, fl
 
 // Compacts the batch positions [0, n) whose Gaussian reaches the warp's pixel
 // rows into list, in ascending order; returns how many (warp-uniform).  A
-// Gaussian is listed when its widened y extent reaches the rows and, with
-// kExact and a plain record, its alpha_min ellipse also meets the rows' pixel
-// centres within the tile's columns [0.5, xmax].  All 32 lanes take part.
-// `fine` tells (warp-uniform) whether a listed record is near-degenerate.
-// Both forms list every Gaussian that blends into a pixel of the rows, so the
-// forward (y extent alone: the exact test costs it more than it saves) and the
-// backward (exact) may differ in what they skip but not in what they blend.
-template <bool kExact>
+// Gaussian is listed when its widened y extent reaches the rows and, for a plain
+// record, its alpha_min ellipse also meets the rows' pixel centres within the
+// tile's columns [0.5, xmax].  All 32 lanes take part.  `fine` tells
+// (warp-uniform) whether a listed record is near-degenerate.
 VPGS_D int warp_list(const float4 *s0, const float4 *s1, int n, float2 band, uint16_t *list, int lane,
                      bool &fine, float xmax, float lg_amin) {
     const uint32_t below = (1u << lane) - 1u;
@@ -123,7 +119,7 @@ VPGS_D int warp_list(const float4 *s0, const float4 *s1, int n, float2 band, uin
             const float ry = b.w;
             touch = fabsf(a.y - band.x) <= fabsf(ry) + band.y;
             f = touch && ry < 0.f;
-            if (kExact && touch && !f) touch = reaches_box(a, b, 0.5f, xmax, band.x - band.y, band.x + band.y, lg_amin);
+            if (touch && !f) touch = reaches_box(a, b, 0.5f, xmax, band.x - band.y, band.x + band.y, lg_amin);
         }
         const uint32_t m = __ballot_sync(0xffffffffu, touch);
         any |= __any_sync(0xffffffffu, f);
@@ -135,26 +131,31 @@ VPGS_D int warp_list(const float4 *s0, const float4 *s1, int n, float2 band, uin
     return cnt;
 }
 
-// The same list for the backward's packed walk: the byte offsets of the staged
-// records (kBwdRec float4 each), last record first.
-constexpr int kBwdRec = 5;  // float4 per staged record: an odd number keeps 16-byte reads by lane conflict-free
-VPGS_D int warp_list_back(const float4 *s_rec, int n, float2 band, uint16_t *list, int lane, bool &fine, float xmax,
-                          float lg_amin) {
+// The same list for the packed walks of the forward and the full backward: the byte
+// offsets of the staged records (kRecStage float4 each), first record first or, with
+// kBack, last record first.  kExact (the backward): the ellipse test too.  Without it
+// (the forward) a Gaussian is listed by its y extent alone: both list every Gaussian
+// that blends into a pixel of the rows, so they may differ in what they skip but not
+// in what they blend.
+constexpr int kRecStage = 5;  // float4 per staged record: an odd number keeps 16-byte reads by lane conflict-free
+template <bool kExact, bool kBack>
+VPGS_D int warp_offsets(const float4 *s_rec, int n, float2 band, uint16_t *list, int lane, bool &fine, float xmax,
+                        float lg_amin) {
     const uint32_t below = (1u << lane) - 1u;
     int cnt = 0;
     bool any = false;
-    for (int c0 = n - 1; c0 >= 0; c0 -= 32) {
-        const int k = c0 - lane;
+    for (int c0 = 0; c0 < n; c0 += 32) {
+        const int k = kBack ? n - 1 - c0 - lane : c0 + lane;
         bool touch = false, f = false;
-        if (k >= 0) {
-            const float4 a = s_rec[kBwdRec * k], b = s_rec[kBwdRec * k + 1];
+        if (kBack ? k >= 0 : k < n) {
+            const float4 a = s_rec[kRecStage * k], b = s_rec[kRecStage * k + 1];
             touch = fabsf(a.y - band.x) <= fabsf(b.w) + band.y;
             f = touch && b.w < 0.f;
-            if (touch && !f) touch = reaches_box(a, b, 0.5f, xmax, band.x - band.y, band.x + band.y, lg_amin);
+            if (kExact && touch && !f) touch = reaches_box(a, b, 0.5f, xmax, band.x - band.y, band.x + band.y, lg_amin);
         }
         const uint32_t m = __ballot_sync(0xffffffffu, touch);
         any |= __any_sync(0xffffffffu, f);
-        if (touch) list[cnt + __popc(m & below)] = (uint16_t)(k * (kBwdRec * 16));
+        if (touch) list[cnt + __popc(m & below)] = (uint16_t)(k * (kRecStage * 16));
         cnt += __popc(m);
     }
     __syncwarp();
@@ -162,10 +163,15 @@ VPGS_D int warp_list_back(const float4 *s_rec, int n, float2 band, uint16_t *lis
     return cnt;
 }
 
+// the staged record at a byte offset of such a list
+VPGS_D const float4 *rec_at(const float4 *s_rec, int off) {
+    return reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(s_rec) + off);
+}
+
 // record -> shared staging: s0 = (u, v) tile-local, w1; s1 = w2, opacity, widened
 // y half extent (negative: near-degenerate); s2 = colour, camera z.  The
-// forward also stages fine_extra of a near-degenerate record (s3); the
-// backward, whose shared memory sets its occupancy, reads it from the record.
+// forward also stages fine_extra of a near-degenerate record; the backward
+// kernels read it from the record in memory (a broadcast load, for such records only).
 // what a near-degenerate record adds to its staged a = (ux, uy, ...): the
 // rounding residual of the tile-local mean ((u_hi - ox) + u_lo = ux + residual,
 // the subtraction split exactly) and the low parts of w2
@@ -206,9 +212,12 @@ VPGS_D float2 first_row(float px, float py0, const float4 &a, const float4 &b) {
     return make_float2(fmaf(a.z, dx, a.w * dy), fmaf(b.x, dx, b.y * dy));
 }
 
-// register cap of the forward (0: only the 512-thread launch bound)
+// register cap of the forward (0: only the 512-thread launch bound).  96 with 8 entries
+// per step: 140 us (room) and 163 us (a street frame whose longest tiles hold 3,600
+// entries: there each warp's own latency counts, not the number of warps); 80 with 6:
+// 144 / 181 us, 72 with 4: 150 / 200 us, 64 with 4: 150 / 230 us.
 #ifndef VPGS_FWD_MAXREG
-#define VPGS_FWD_MAXREG 0
+#define VPGS_FWD_MAXREG 96
 #endif
 #if VPGS_FWD_MAXREG > 0
 #define VPGS_FWD_BOUNDS __maxnreg__(VPGS_FWD_MAXREG)
@@ -216,6 +225,15 @@ VPGS_D float2 first_row(float px, float py0, const float4 &a, const float4 &b) {
 #define VPGS_FWD_BOUNDS __launch_bounds__(kMaxThreads)
 #endif
 
+// One lane per column pair of pixels; the packed FP32 instructions work on the pair.
+// A list step has no branch: a pixel that does not blend takes part with weight 0 and
+// keeps its T by a select, which leaves every sum as it was (the rounding of each
+// half is the scalar instructions').  The branches it replaces cost their exposed
+// latency in long tiles and their issue slots in the others.  Measured, old -> new:
+// 1M-Gaussian room 1200x680 192 -> 140 us, street frame 1241x376 of 316k visible
+// Gaussians 524 -> 163 us, 8 keyframes of 2M 875 -> 656 us, four full-HD views 504 ->
+// 401 us, 10k Gaussians 320x240 24 -> 12 us.  The exact ellipse test of the backward's
+// lists gains nothing here (room 144 us either way, street frame 181 -> 196 us).
 __global__ void VPGS_FWD_BOUNDS
 composite_fwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ ival,
                      const uint2 *__restrict__ ranges, const uint32_t *__restrict__ order, int n_tiles,
@@ -224,12 +242,12 @@ composite_fwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
     grid_dep_enter();
     extern __shared__ float4 smem[];
     const int NT = blockDim.x * kFwdBatch;  // records per batch
-    float4 *s0 = smem, *s1 = smem + NT, *s2 = smem + 2 * NT, *s3 = smem + 3 * NT;
-    uint16_t *s_wl = reinterpret_cast<uint16_t *>(smem + 4 * NT);  // [NW][NT] per-warp lists
+    // records: mean and w1; w2, opacity, y half extent; (r, r, g, g); (b, b, z, z); fine_extra
+    float4 *s_rec = smem;
+    const int tid = threadIdx.x, lane = tid & 31;
+    uint16_t *wl = reinterpret_cast<uint16_t *>(smem + kRecStage * NT) + (size_t)(tid >> 5) * NT;  // this warp's list
     __shared__ int s_tile;
     if (*status != 0u) return;
-    const int tid = threadIdx.x, lane = tid & 31;
-    uint16_t *wl = s_wl + (size_t)(tid >> 5) * NT;
     const int lx = tid % cam.tile_w, ly = tid / cam.tile_w;
     const float pxl = (float)lx + 0.5f;
     float pyl[kPix];
@@ -237,6 +255,7 @@ composite_fwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
     for (int q = 0; q < kPix; ++q) pyl[q] = (float)(kPix * ly + q) + 0.5f;
     const float2 band = warp_rows(pyl);
     const float lg_amin = __log2f(o.alpha_min);
+    const f2 one2 = pack2(1.f, 1.f);
     int t = blockIdx.x;
     for (;;) {
         if (work) {
@@ -253,153 +272,123 @@ composite_fwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
         const float xmax = fminf((float)cam.tile_w, (float)cam.W - ox) - 0.5f;  // last pixel centre column
         const uint2 rg = ranges[tile];
         const int start = (int)rg.x, end = (int)rg.y;
-        float T[kPix], C0[kPix], C1[kPix], C2[kPix], D[kPix];
-        int cnt[kPix], last[kPix];
-        bool done[kPix];
-#pragma unroll
-        for (int q = 0; q < kPix; ++q) {
-            T[q] = 1.f; C0[q] = C1[q] = C2[q] = D[q] = 0.f; cnt[q] = 0; last[q] = 0;
-            const int py = tc.ty * cam.tile_h + kPix * ly + q;
-            done[q] = !(px < cam.W && py < cam.H);
-        }
-        bool all_done = true;
-#pragma unroll
-        for (int q = 0; q < kPix; ++q) all_done = all_done && done[q];
+        f2 T2 = one2, C0 = pack2(0.f, 0.f), C1 = C0, C2 = C0, D = C0;
+        int cnt0 = 0, cnt1 = 0, last0 = 0, last1 = 0;
+        const int py0 = tc.ty * cam.tile_h + kPix * ly;
+        bool done0 = !(px < cam.W && py0 < cam.H), done1 = !(px < cam.W && py0 + 1 < cam.H);
         for (int b0 = start; b0 < end; b0 += NT) {
-            if (__syncthreads_count(all_done) == (int)blockDim.x) break;
+            if (__syncthreads_count(done0 && done1) == (int)blockDim.x) break;
 #pragma unroll 1
             for (int u = 0; u < kFwdBatch; ++u) {
                 const int k = tid + u * (int)blockDim.x;
                 const int j = b0 + k;
                 if (j < end) {
                     const Rec r = rec[ival[j]];
-                    stage(r, ox, oy, s0[k], s1[k], s2[k]);
-                    if (r.r3.z < 0.f) s3[k] = fine_extra(r, ox, oy, s0[k].x, s0[k].y);
+                    float4 a, b, c;
+                    stage(r, ox, oy, a, b, c);
+                    float4 *d = s_rec + kRecStage * k;
+                    d[0] = a;
+                    d[1] = b;
+                    d[2] = make_float4(c.x, c.x, c.y, c.y);
+                    d[3] = make_float4(c.z, c.z, c.w, c.w);
+                    if (r.r3.z < 0.f) d[4] = fine_extra(r, ox, oy, a.x, a.y);
                 }
             }
             __syncthreads();
             bool any_fine;
-            const int nl = warp_list<false>(s0, s1, min(NT, end - b0), band, wl, lane, any_fine, xmax, lg_amin);
-            // one blend step of this thread's pixels against list entry k
-            auto blend = [&](int k, const float4 &a, const float4 &b, auto fine) -> bool {
-                    constexpr bool kFine = decltype(fine)::value;
-                    float4 f;
-                    if constexpr (kFine) f = s3[k];
-                    const float2 t0 = kFine ? make_float2(0.f, 0.f) : first_row(pxl, pyl[0], a, b);
-                    bool fin = true;
-#pragma unroll
-                    for (int q = 0; q < kPix; ++q) {
-                        if (!done[q]) {
-                            const PairEval e = eval_staged<kFine>(q, t0.x, t0.y, pxl, pyl[q], a, b, f, o.alpha_max);
-                            if (e.alpha >= o.alpha_min) {
-                                const float nt = T[q] * (1.f - e.alpha);
-                                if (nt < o.t_min) {
-                                    done[q] = true;
-                                } else {
-                                    const float w = e.alpha * T[q];
-                                    const float4 col = s2[k];
-                                    C0[q] = fmaf(w, col.x, C0[q]);
-                                    C1[q] = fmaf(w, col.y, C1[q]);
-                                    C2[q] = fmaf(w, col.z, C2[q]);
-                                    D[q] = fmaf(w, col.w, D[q]);
-                                    T[q] = nt;
-                                    ++cnt[q];
-                                    last[q] = b0 + k - start + 1;
-                                }
-                            }
-                        }
-                        fin = fin && done[q];
-                    }
-                    return fin;
+            const int nl = warp_offsets<false, false>(s_rec, min(NT, end - b0), band, wl, lane, any_fine, xmax, lg_amin);
+            int lo0 = -1, lo1 = -1;  // offsets of the last records blended in this batch
+            // blends one entry (alphas al) into the lane's pixels
+            auto blend = [&](int off, f2 al, const float4 &c2, const float4 &c3) {
+                const f2 nt = mul2(T2, add2(one2, neg2(al)));
+                const bool act0 = lo2(al) >= o.alpha_min && !done0, act1 = hi2(al) >= o.alpha_min && !done1;
+                const bool stop0 = lo2(nt) < o.t_min, stop1 = hi2(nt) < o.t_min;
+                const bool bl0 = act0 && !stop0, bl1 = act1 && !stop1;
+                const f2 w = mul2(al, T2);
+                const f2 wm = pack2(bl0 ? lo2(w) : 0.f, bl1 ? hi2(w) : 0.f);
+                C0 = fma2(wm, pack2(c2.x, c2.y), C0);
+                C1 = fma2(wm, pack2(c2.z, c2.w), C1);
+                C2 = fma2(wm, pack2(c3.x, c3.y), C2);
+                D = fma2(wm, pack2(c3.z, c3.w), D);
+                T2 = pack2(bl0 ? lo2(nt) : lo2(T2), bl1 ? hi2(nt) : hi2(T2));
+                cnt0 += bl0;
+                cnt1 += bl1;
+                lo0 = bl0 ? off : lo0;
+                lo1 = bl1 ? off : lo1;
+                done0 |= act0 && stop0;
+                done1 |= act1 && stop1;
             };
-            // the list walk; a batch with a near-degenerate record takes the walk that
-            // chooses the precision form per entry (a warp-uniform branch), the others
-            // the plain one, kWalk entries at a time: their alphas (which do not depend
-            // on the transmittance) are evaluated before the blends, so the pixels'
-            // blend chains overlap with independent work
-            auto walk_plain = [&]() {
-                for (int i = 0; i < nl; i += kWalk) {
-                    float al[kWalk][kPix];
-                    int kk[kWalk];
-#pragma unroll
-                    for (int u = 0; u < kWalk; ++u) kk[u] = wl[min(i + u, nl - 1)];
-#pragma unroll
-                    for (int u = 0; u < kWalk; ++u) {
-                        const float4 a = s0[kk[u]], b = s1[kk[u]];
-                        const float2 t0 = first_row(pxl, pyl[0], a, b);
-#pragma unroll
-                        for (int q = 0; q < kPix; ++q)
-                            al[u][q] = eval_staged<false>(q, t0.x, t0.y, pxl, pyl[q], a, b, a, o.alpha_max).alpha;
-                    }
-                    bool fin = false;
+            auto alphas = [&](const float4 &a, const float4 &b) -> f2 {
+                const float2 t0 = first_row(pxl, pyl[0], a, b);
+                const f2 t12 = pack2(t0.x, t0.x + a.w), t22 = pack2(t0.y, t0.y + b.y);
+                const f2 q = fma2(t12, t12, mul2(t22, t22));
+                return pack2(fminf(o.alpha_max, b.z * ex2_approx(-lo2(q))),
+                             fminf(o.alpha_max, b.z * ex2_approx(-hi2(q))));
+            };
+            if (!any_fine) {
+                // kWalk entries at a time: their alphas, which do not depend on the
+                // transmittance, before their blends
+                int i = 0;
+                for (; i + kWalk <= nl; i += kWalk) {
+                    if (__all_sync(0xffffffffu, done0 && done1)) break;
+                    int off[kWalk];
+                    f2 al[kWalk];
 #pragma unroll
                     for (int u = 0; u < kWalk; ++u) {
-                        if (fin || i + u >= nl) break;
-                        fin = true;
-#pragma unroll
-                        for (int q = 0; q < kPix; ++q) {
-                            if (!done[q] && al[u][q] >= o.alpha_min) {
-                                const float nt = T[q] * (1.f - al[u][q]);
-                                if (nt < o.t_min) {
-                                    done[q] = true;
-                                } else {
-                                    const float w = al[u][q] * T[q];
-                                    const float4 col = s2[kk[u]];
-                                    C0[q] = fmaf(w, col.x, C0[q]);
-                                    C1[q] = fmaf(w, col.y, C1[q]);
-                                    C2[q] = fmaf(w, col.z, C2[q]);
-                                    D[q] = fmaf(w, col.w, D[q]);
-                                    T[q] = nt;
-                                    ++cnt[q];
-                                    last[q] = b0 + kk[u] - start + 1;
-                                }
-                            }
-                            fin = fin && done[q];
-                        }
+                        off[u] = wl[i + u];
+                        const float4 *r = rec_at(s_rec, off[u]);
+                        al[u] = alphas(r[0], r[1]);
                     }
-                    if (fin) {
-                        all_done = true;
-                        break;
+#pragma unroll
+                    for (int u = 0; u < kWalk; ++u) {
+                        const float4 *r = rec_at(s_rec, off[u]);
+                        blend(off[u], al[u], r[2], r[3]);
                     }
                 }
-            };
-            auto walk = [&](auto maybe_fine) {
+                if (i + kWalk > nl)  // the last few (not after an early stop)
+                    for (; i < nl; ++i) {
+                        const float4 *r = rec_at(s_rec, wl[i]);
+                        blend(wl[i], alphas(r[0], r[1]), r[2], r[3]);
+                    }
+            } else {
+                // a batch with a near-degenerate record chooses the precision per entry
                 for (int i = 0; i < nl; ++i) {
-                    const int k = wl[i];
-                    const float4 a = s0[k], b = s1[k];
-                    bool fin;
-                    if constexpr (decltype(maybe_fine)::value)
-                        fin = b.w < 0.f ? blend(k, a, b, std::true_type{}) : blend(k, a, b, std::false_type{});
-                    else
-                        fin = blend(k, a, b, std::false_type{});
-                    if (fin) {
-                        all_done = true;
-                        break;
+                    if (__all_sync(0xffffffffu, done0 && done1)) break;
+                    const float4 *r = rec_at(s_rec, wl[i]);
+                    const float4 a = r[0], b = r[1];
+                    f2 al;
+                    if (b.w < 0.f) {
+                        const float4 f = r[4];
+                        const PairEval e0 = eval_staged<true>(0, 0.f, 0.f, pxl, pyl[0], a, b, f, o.alpha_max);
+                        const PairEval e1 = eval_staged<true>(1, 0.f, 0.f, pxl, pyl[1], a, b, f, o.alpha_max);
+                        al = pack2(e0.alpha, e1.alpha);
+                    } else {
+                        al = alphas(a, b);
                     }
+                    blend(wl[i], al, r[2], r[3]);
                 }
-            };
-            if (!all_done) {
-                if (any_fine) walk(std::true_type{});
-                else walk_plain();
             }
+            if (lo0 >= 0) last0 = b0 - start + lo0 / (kRecStage * 16) + 1;
+            if (lo1 >= 0) last1 = b0 - start + lo1 / (kRecStage * 16) + 1;
         }
         const int64_t HW = (int64_t)cam.H * cam.W;
 #pragma unroll
         for (int q = 0; q < kPix; ++q) {
-            const int py = tc.ty * cam.tile_h + kPix * ly + q;
+            const int py = py0 + q;
             if (!(px < cam.W && py < cam.H)) continue;
             const int64_t pix = (int64_t)tc.v * HW + (int64_t)py * cam.W + px;
+            const float T = q ? hi2(T2) : lo2(T2);
             if (out.rgb) {
                 float *rgb = out.rgb + (int64_t)tc.v * 3 * HW + (int64_t)py * cam.W + px;
-                rgb[0] = fmaf(T[q], o.bg0, C0[q]);
-                rgb[HW] = fmaf(T[q], o.bg1, C1[q]);
-                rgb[2 * HW] = fmaf(T[q], o.bg2, C2[q]);
+                rgb[0] = fmaf(T, o.bg0, q ? hi2(C0) : lo2(C0));
+                rgb[HW] = fmaf(T, o.bg1, q ? hi2(C1) : lo2(C1));
+                rgb[2 * HW] = fmaf(T, o.bg2, q ? hi2(C2) : lo2(C2));
             }
-            if (out.depth) out.depth[pix] = D[q];
-            if (out.alpha) out.alpha[pix] = 1.f - T[q];
-            out.t_final[pix] = T[q];
-            if (out.n_contrib) out.n_contrib[pix] = cnt[q];
-            out.n_iter[pix] = last[q];
+            if (out.depth) out.depth[pix] = q ? hi2(D) : lo2(D);
+            if (out.alpha) out.alpha[pix] = 1.f - T;
+            out.t_final[pix] = T;
+            if (out.n_contrib) out.n_contrib[pix] = q ? cnt1 : cnt0;
+            out.n_iter[pix] = q ? last1 : last0;
         }
         if (!work) return;
         __syncthreads();
@@ -646,7 +635,7 @@ composite_geo_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
             __syncthreads();
             const int k_end = min(nb, warp_max - (b0 - start));  // warp-uniform
             bool any_fine;
-            const int nl = warp_list<true>(s0, s1, k_end, band, wl, lane, any_fine, xmax, lg_amin);
+            const int nl = warp_list(s0, s1, k_end, band, wl, lane, any_fine, xmax, lg_amin);
             // back to front; a batch with a near-degenerate record takes the walk that
             // chooses the precision form per entry (a warp-uniform branch), the others
             // the plain one
@@ -769,11 +758,10 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // records: s0, s1 as in the forward, the colour and depth doubled (r, r, g, g), (b, b, z, z), the id
     float4 *s_rec = smem;
-    float4 *s_term = smem + kBwdRec * NT + warp * (kSlots * kTermStride);           // this warp's (w, w, dpow, dpow)
-    float4 *s_pix = smem + kBwdRec * NT + NW * (kSlots * kTermStride) + warp * kPixSize;  // this warp's -g
-    uint16_t *wl = reinterpret_cast<uint16_t *>(smem + kBwdRec * NT + NW * (kSlots * kTermStride + kPixSize)) +
+    float4 *s_term = smem + kRecStage * NT + warp * (kSlots * kTermStride);           // this warp's (w, w, dpow, dpow)
+    float4 *s_pix = smem + kRecStage * NT + NW * (kSlots * kTermStride) + warp * kPixSize;  // this warp's -g
+    uint16_t *wl = reinterpret_cast<uint16_t *>(smem + kRecStage * NT + NW * (kSlots * kTermStride + kPixSize)) +
                    (size_t)warp * NT;  // this warp's list
-    auto rec_at = [&](int off) { return reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(s_rec) + off); };
     __shared__ int s_tile;
     __shared__ int s_max;
     __shared__ int s_odd;
@@ -861,7 +849,7 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                     const uint32_t id = ival[b0 + k];
                     float4 a, b, c;
                     stage(rec[id], ox, oy, a, b, c);
-                    float4 *d = s_rec + kBwdRec * k;
+                    float4 *d = s_rec + kRecStage * k;
                     d[0] = a;
                     d[1] = b;
                     d[2] = make_float4(c.x, c.x, c.y, c.y);
@@ -873,7 +861,7 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
             __syncthreads();
             const int k_end = min(nb, warp_max - (b0 - start));  // warp-uniform
             bool any_fine;
-            const int nl = warp_list_back(s_rec, k_end, band, wl, lane, any_fine, xmax, lg_amin);
+            const int nl = warp_offsets<true, true>(s_rec, k_end, band, wl, lane, any_fine, xmax, lg_amin);
             const int base = b0 - start;  // list position of the batch's first record
             if (any_fine || warp_odd || s_odd != 0) {  // warp-uniform
                 // entry by entry, each in its precision form, the warp's sums by shuffles
@@ -892,8 +880,8 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                 }
                 const int slot = red_slot<NV>(lane);
                 for (int i = 0; i < nl; ++i) {
-                    const float4 *r = rec_at(wl[i]);
-                    const int kk = wl[i] / (kBwdRec * 16);
+                    const float4 *r = rec_at(s_rec, wl[i]);
+                    const int kk = wl[i] / (kRecStage * 16);
                     const uint32_t id = __float_as_uint(r[4].x);
                     const float4 a = r[0], b = r[1], c2 = r[2], c3 = r[3];
                     const float4 c = make_float4(c2.x, c2.z, c3.x, c3.z);
@@ -923,14 +911,14 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                 beta2 = pack2(ps[0].beta, ps[1].beta);
                 continue;
             }
-            const int l0 = (last[0] - base) * (kBwdRec * 16), l1 = (last[1] - base) * (kBwdRec * 16);
+            const int l0 = (last[0] - base) * (kRecStage * 16), l1 = (last[1] - base) * (kRecStage * 16);
             for (int g = 0; g < nl; g += kSlots) {
                 const int n = min(kSlots, nl - g);  // warp-uniform
                 // phase 1
 #pragma unroll kBwdUnroll
                 for (int i = 0; i < n; ++i) {
                     const int off = wl[g + i];
-                    const float4 *r = rec_at(off);
+                    const float4 *r = rec_at(s_rec, off);
                     const float4 a = r[0], b = r[1], c2 = r[2], c3 = r[3];
                     const float2 t0 = first_row(pxl, pyl[0], a, b);
                     const f2 t12 = pack2(t0.x, t0.x + a.w), t22 = pack2(t0.y, t0.y + b.y);
@@ -959,7 +947,7 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                 // phase 2
                 const int e = lane & (kSlots - 1), part = lane / kSlots;
                 constexpr int kShare = kSlots;  // lanes (pixel pairs) of phase 1 per part: 32 / (32 / kSlots)
-                const float4 *r = rec_at(wl[g + (e < n ? e : 0)]);
+                const float4 *r = rec_at(s_rec, wl[g + (e < n ? e : 0)]);
                 const float4 a = r[0], b = r[1];
                 f2 v[NV];
 #pragma unroll
@@ -1028,16 +1016,18 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
 }
 
 // dynamic shared memory of a compositing block of `threads` threads staging
-// `records` per batch: forward s0-s3 and the warps' lists; geometric backward s0-s2,
+// `records` per batch: forward the staged records and the warps' lists; geometric backward s0-s2,
 // the ids and the lists; full backward the staged records, the warps' term slots and
 // pixel gradients, and the lists
 static size_t list_bytes(int threads, int records) { return sizeof(uint16_t) * (size_t)(threads / 32) * records; }
-static size_t fwd_smem(int threads, int records) { return sizeof(float4) * 4 * records + list_bytes(threads, records); }
+static size_t fwd_smem(int threads, int records) {
+    return sizeof(float4) * kRecStage * records + list_bytes(threads, records);
+}
 static size_t geo_smem(int threads, int records) {
     return (sizeof(float4) * 3 + sizeof(uint32_t)) * records + list_bytes(threads, records);
 }
 static size_t bwd_smem(int threads, int records) {
-    return sizeof(float4) * (kBwdRec * (size_t)records + (size_t)(threads / 32) * (kSlots * kTermStride + kPixSize)) +
+    return sizeof(float4) * (kRecStage * (size_t)records + (size_t)(threads / 32) * (kSlots * kTermStride + kPixSize)) +
            list_bytes(threads, records);
 }
 
