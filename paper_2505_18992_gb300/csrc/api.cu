@@ -78,7 +78,7 @@ bool make_layout(int64_t N, int V, const vpgs_camera *cam, const vpgs_render_opt
     L.off_ranges = take(sizeof(uint2) * (size_t)V * L.T);
     L.off_sort_hist = take(2 * 4 * kRadix * 4);
     const int64_t look_a = 4 * sort_blocks(VN1, kDepthSortItems);
-    const int64_t look_b = (int64_t)std::max(np_tile, 1) * sort_blocks(L.M_cap, kTileSortItems);
+    const int64_t look_b = (int64_t)std::max(np_tile, 1) * sort_dpt(L.tile_bits) * sort_blocks(L.M_cap, kTileSortItems);
     L.sort_blocks_max = look_a > look_b ? look_a : look_b;
     L.off_sort_look = take(4 * kRadix * (size_t)look_a);
     L.off_sort_look_t = take(4 * kRadix * (size_t)look_b);

@@ -35,7 +35,35 @@ struct GaussGrad {
 
 int device_sm_count();
 
+// Which form the binning of a call takes (render_bin.cu): its general one, or for small
+// calls the ranking by comparison, with tile lists by selection (kSmallLists) or by the
+// general emission and sort (kSmallRank).  The small forms cost pairs^2 and pairs x tiles;
+// the lines lie where their measured forward met the general one's with every pair
+// visible (us, small / general): 12,288 pairs x 300 tiles 65 / 75, x 1,200 85 / 94,
+// x 1,900 99 / 96; 12,000 pairs by rank alone 133 / 117; 5,000 pairs x 300 tiles 33 / 65,
+// 1,000 22 / 52.
+enum BinForm { kGeneralBin, kSmallRank, kSmallLists };
+constexpr int64_t kSmallPairs = 12288;       // (below 2^14: a pair fits 16 bits beside its view)
+constexpr int64_t kSmallRankPairs = 6144;
+constexpr int64_t kSmallProduct = 15000000;  // pairs x tiles
+inline BinForm bin_form(const RenderLayout &L) {
+    const int64_t tiles = (int64_t)L.V * L.T;
+    // (four bytes of a tile rectangle, 16 bits of a view)
+    if (L.VN <= kSmallPairs && L.VN * tiles <= kSmallProduct && L.tiles_x <= 256 && L.tiles_y <= 256 && L.V <= 65535)
+        return kSmallLists;
+    return L.VN <= kSmallRankPairs ? kSmallRank : kGeneralBin;
+}
 
+// The visible (view, Gaussian) pairs of a small call, in any order, as the projection
+// appends them: depth key, tile count, pair index.  They lie in the depth sort's
+// buffers, which such a call does not use; NULL otherwise.
+struct SmallList {
+    uint32_t *key, *cnt, *pair;
+};
+inline SmallList small_list(const RenderWs &ws, const RenderLayout &L) {
+    if (bin_form(L) == kGeneralBin) return SmallList{nullptr, nullptr, nullptr};
+    return SmallList{ws.dkey[0], ws.dval[0], ws.dval[1]};
+}
 
 // render_pre.cu
 // First launches of a render call: the prepare kernel (zeroes status, counters
@@ -59,6 +87,8 @@ cudaError_t build_tile_lists(const GaussIn &g, int V, const CamParams &cam, cons
 // list steps, most first (ws.tile_work, ws.tile_order).
 cudaError_t order_tiles_by_steps(const RenderWs &ws, const int32_t *n_iter, int V, const CamParams &cam,
                                  cudaStream_t s);
+// Whether calls of n_tiles tiles use a launch order (ws.tile_order) at all.
+bool tiles_ordered(int n_tiles, const CamParams &cam);
 // Which ival buffer build_tile_lists leaves the tile lists in (host only, no launch).
 int tile_list_buffer(const RenderLayout &L);
 

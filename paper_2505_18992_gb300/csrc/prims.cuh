@@ -8,6 +8,8 @@
 // still bounds-checked.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "profiler.h"
 
@@ -256,7 +258,8 @@ constexpr uint32_t kSFlagAgg = 1u << 30;
 constexpr uint32_t kSFlagPre = 2u << 30;
 constexpr uint32_t kSValMask = (1u << 30) - 1u;
 
-template <int ITEMS>
+// DPT: digits per thread (1: digits of up to 8 bits, 2: up to 9)
+template <int ITEMS, int DPT>
 static __global__ void __launch_bounds__(kSortThreads)
 radix_onesweep_kernel(const uint32_t *__restrict__ key_in, const uint32_t *__restrict__ val_in,
                       uint32_t *__restrict__ key_out, uint32_t *__restrict__ val_out,
@@ -268,10 +271,14 @@ radix_onesweep_kernel(const uint32_t *__restrict__ key_in, const uint32_t *__res
     constexpr int kWarps = kSortThreads / kWarp;
     constexpr int kSeg = kWarp * ITEMS;  // contiguous items per warp
     constexpr int kTile = kSortThreads * ITEMS;
-    static_assert(kSortThreads == kRadix, "one thread per digit");
-    __shared__ uint32_t s_cnt[kWarps][kRadix];
+    constexpr int kDigits = kRadix * DPT;
+    static_assert(kSortThreads == kRadix, "a thread takes DPT consecutive digits");
+    // (16-bit counts, a tile holds at most 4,096 keys, keep 512 digits within 48 KB)
+    using Count = typename std::conditional<DPT == 1, uint32_t, uint16_t>::type;
+    static_assert(DPT == 1 || kTile < 65536, "a tile's counts fit 16 bits");
+    __shared__ Count s_cnt[kWarps][kDigits];
     __shared__ uint32_t s_glob[kRadix];
-    __shared__ uint32_t s_dstart[kRadix], s_gbase[kRadix], s_wsum[kWarps];
+    __shared__ uint32_t s_dstart[kDigits], s_gbase[kDigits], s_wsum[kWarps];
     __shared__ uint32_t s_key[kTile], s_val[kTile];
     __shared__ uint32_t s_bid;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -281,30 +288,33 @@ radix_onesweep_kernel(const uint32_t *__restrict__ key_in, const uint32_t *__res
     const uint32_t mask = (1u << pass.bits) - 1u;
 
     // global exclusive digit offsets of this pass (every block recomputes them)
-    if (tid < kRadix) {
-        // 256 threads: inclusive scan via shared memory in two levels of warps
-        uint32_t h = pass_hist[tid];
-        uint32_t x = h;
+    uint32_t glob_excl[DPT], hist_sum = 0;
+#pragma unroll
+    for (int e = 0; e < DPT; ++e) {
+        glob_excl[e] = hist_sum;
+        hist_sum += pass_hist[tid * DPT + e];
+    }
+    {
+        // inclusive scan of the threads' sums in two levels of warps
+        uint32_t x = hist_sum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
         s_glob[tid] = x;  // inclusive within warp
-    }
-    __syncthreads();
-    uint32_t glob_excl = 0;
-    if (tid < kRadix) {
-        uint32_t add = 0;
+        __syncthreads();
+        uint32_t add = x - hist_sum;
         for (int w = 0; w < warp; ++w) add += s_glob[w * 32 + 31];
-        glob_excl = s_glob[tid] - pass_hist[tid] + add;
+#pragma unroll
+        for (int e = 0; e < DPT; ++e) glob_excl[e] += add;
     }
 
     // tiles in ticket order until they run out (the grid is sized to what fits
     // on the GPU at once; a tile only waits on lower tickets, held by running blocks)
     for (;;) {
     if (tid == 0) s_bid = atomicAdd(ticket, 1u);
-    for (int i = tid; i < kWarps * kRadix; i += kSortThreads) (&s_cnt[0][0])[i] = 0;
+    for (int i = tid; i < kWarps * kDigits; i += kSortThreads) (&s_cnt[0][0])[i] = 0;
     __syncthreads();
     const int64_t bid = s_bid;
     const int64_t base = bid * (int64_t)(kSortThreads * ITEMS);
@@ -319,22 +329,27 @@ radix_onesweep_kernel(const uint32_t *__restrict__ key_in, const uint32_t *__res
         bool ok = i < n;
         k[s] = ok ? key_in[i] : 0u;
         v[s] = ok ? val_in[i] : 0u;
-        d[s] = ok ? ((k[s] >> pass.shift) & mask) : (kRadix + lane);  // sentinel never matches
+        d[s] = ok ? ((k[s] >> pass.shift) & mask) : (kDigits + lane);  // sentinel never matches
     }
     // per-warp digit counts
 #pragma unroll
     for (int s = 0; s < ITEMS; ++s) {
-        const uint32_t m = match_digit(d[s], d[s] < kRadix, pass.bits, lane);
-        if (d[s] < kRadix && (m & lanemask_lt()) == 0) s_cnt[warp][d[s]] += __popc(m);
+        const uint32_t m = match_digit(d[s], d[s] < kDigits, pass.bits, lane);
+        if (d[s] < kDigits && (m & lanemask_lt()) == 0) s_cnt[warp][d[s]] += (Count)__popc(m);
         __syncwarp();
     }
     __syncthreads();
-    // block count per digit and its block-local exclusive start (kRadix == threads)
-    uint32_t c = 0;
+    // block count per digit and its block-local exclusive start
+    uint32_t c[DPT], csum = 0;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) c += s_cnt[w][tid];
+    for (int e = 0; e < DPT; ++e) {
+        c[e] = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) c[e] += s_cnt[w][tid * DPT + e];
+        csum += c[e];
+    }
     {
-        uint32_t x = c;
+        uint32_t x = csum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
@@ -342,18 +357,23 @@ radix_onesweep_kernel(const uint32_t *__restrict__ key_in, const uint32_t *__res
         }
         if (lane == 31) s_wsum[warp] = x;
         __syncthreads();
-        uint32_t add = 0;
+        uint32_t add = x - csum;
         for (int w = 0; w < warp; ++w) add += s_wsum[w];
-        s_dstart[tid] = x - c + add;
+#pragma unroll
+        for (int e = 0; e < DPT; ++e) {
+            s_dstart[tid * DPT + e] = add;
+            add += c[e];
+        }
     }
     // publish, look back over earlier blocks
-    {
+#pragma unroll
+    for (int e = 0; e < DPT; ++e)
+        st_volatile_u32(look + bid * kDigits + tid * DPT + e, (bid == 0 ? kSFlagPre : kSFlagAgg) | c[e]);
+#pragma unroll
+    for (int e = 0; e < DPT; ++e) {
+        const int dg = tid * DPT + e;
         uint32_t excl = 0;
-        uint32_t *my = look + bid * kRadix + tid;
-        if (bid == 0) {
-            st_volatile_u32(my, kSFlagPre | c);
-        } else {
-            st_volatile_u32(my, kSFlagAgg | c);
+        if (bid > 0) {
             // kLookDepth independent loads per step shorten the dependent chain
             constexpr int kLookDepth = VPGS_LOOK_DEPTH;
             int64_t j0 = bid - 1;
@@ -363,7 +383,7 @@ radix_onesweep_kernel(const uint32_t *__restrict__ key_in, const uint32_t *__res
 #pragma unroll
                 for (int i = 0; i < kLookDepth; ++i) {
                     const int64_t j = j0 - i;
-                    w[i] = j >= 0 ? ld_volatile_u32(look + j * kRadix + tid) : kSFlagPre;
+                    w[i] = j >= 0 ? ld_volatile_u32(look + j * kDigits + dg) : kSFlagPre;
                 }
 #pragma unroll
                 for (int i = 0; i < kLookDepth; ++i) {
@@ -378,22 +398,22 @@ radix_onesweep_kernel(const uint32_t *__restrict__ key_in, const uint32_t *__res
                             break;
                         }
                         __nanosleep(32);
-                        x = ld_volatile_u32(look + j * kRadix + tid);
+                        x = ld_volatile_u32(look + j * kDigits + dg);
                     }
                     excl += x & kSValMask;
                     if ((x >> 30) == 2) done = true;
                 }
                 j0 -= kLookDepth;
             }
-            st_volatile_u32(my, kSFlagPre | (excl + c));
+            st_volatile_u32(look + bid * kDigits + dg, kSFlagPre | (excl + c[e]));
         }
-        s_gbase[tid] = glob_excl + excl;  // global slot of this block's first key with digit tid
+        s_gbase[dg] = glob_excl[e] + excl;  // global slot of this block's first key with this digit
         // per-warp bases inside the block (block-local digit order)
-        uint32_t run = s_dstart[tid];
+        uint32_t run = s_dstart[dg];
 #pragma unroll
         for (int w = 0; w < kWarps; ++w) {
-            const uint32_t t = s_cnt[w][tid];
-            s_cnt[w][tid] = run;
+            const uint32_t t = s_cnt[w][dg];
+            s_cnt[w][dg] = (Count)run;
             run += t;
         }
     }
@@ -402,15 +422,15 @@ radix_onesweep_kernel(const uint32_t *__restrict__ key_in, const uint32_t *__res
     // order, warps in order
 #pragma unroll
     for (int s = 0; s < ITEMS; ++s) {
-        const uint32_t m = match_digit(d[s], d[s] < kRadix, pass.bits, lane);
+        const uint32_t m = match_digit(d[s], d[s] < kDigits, pass.bits, lane);
         const uint32_t rank = __popc(m & lanemask_lt());
-        if (d[s] < kRadix) {
+        if (d[s] < kDigits) {
             const uint32_t lp = s_cnt[warp][d[s]] + rank;
             s_key[lp] = k[s];
             s_val[lp] = v[s];
         }
         __syncwarp();
-        if (d[s] < kRadix && rank == 0) s_cnt[warp][d[s]] += __popc(m);
+        if (d[s] < kDigits && rank == 0) s_cnt[warp][d[s]] += (Count)__popc(m);
         __syncwarp();
     }
     __syncthreads();
@@ -425,14 +445,23 @@ radix_onesweep_kernel(const uint32_t *__restrict__ key_in, const uint32_t *__res
             val_out[pos] = s_val[i];
         }
     }
-    if (next_look) next_look[bid * kRadix + tid] = 0u;  // the next pass starts from zero
+    if (next_look) {  // the next pass starts from zero
+#pragma unroll
+        for (int e = 0; e < DPT; ++e) next_look[bid * kDigits + tid * DPT + e] = 0u;
+    }
     __syncthreads();  // the next tile reuses the shared arrays
     }
 }
 
-// Split `bits` low key bits starting at `lo` into balanced passes of <= 8 bits.
+// Digits per thread of a sort over `bits` key bits: 2 for 9 bits (257 to 512 tiles), one
+// pass of 9-bit digits instead of two passes, else 1.  A pass costs 7-13 us however few
+// its keys, and one pass of 512 digits takes the look-back words of two of 256.
+inline int sort_dpt(int bits) { return bits == kRadixBits + 1 ? 2 : 1; }
+
+// Split `bits` low key bits starting at `lo` into balanced passes of <= 8 (9: sort_dpt) bits.
 inline int plan_passes(int lo, int bits, SortPass *out) {
-    int np = (bits + kRadixBits - 1) / kRadixBits;
+    const int most = kRadixBits + (sort_dpt(bits) == 2 ? 1 : 0);
+    int np = (bits + most - 1) / most;
     if (np == 0) return 0;
     int base = bits / np, extra = bits % np, s = lo;
     for (int p = 0; p < np; ++p) {
@@ -451,9 +480,9 @@ inline int64_t sort_blocks(int64_t n, int items) {
 // Sort n (<= n_cap, or *n_dev) pairs from (k0, v0) using (k1, v1) as the other
 // buffer.  Returns in *result_in_1 whether the sorted data ended in buffer 1.
 // On entry (the producers of the keys and the render's prepare kernel see to it):
-//   hist   [passes][256] global digit histograms of the n keys;
+//   hist   [passes][256 * sort_dpt(bits)] global digit histograms of the n keys;
 //   ticket [passes] zero;
-//   look   [passes][sort_blocks(n_cap)][256], pass 0's words zero for the tiles
+//   look   [passes][sort_blocks(n_cap)][256 * sort_dpt(bits)], pass 0's words zero for the tiles
 //          that hold keys (each pass clears the next pass's words of its tiles).
 inline cudaError_t radix_sort_pairs(const char *name, uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1,
                                     int64_t n_cap, const uint32_t *n_dev, int lo_bit, int bits,
@@ -465,34 +494,27 @@ inline cudaError_t radix_sort_pairs(const char *name, uint32_t *k0, uint32_t *v0
     *result_in_1 = (np & 1) != 0;
     if (np == 0 || n_cap == 0) return cudaSuccess;
     if (np > 4) return cudaErrorInvalidValue;
-    if (items != 4 && items != 8 && items != 16 && items != 32) return cudaErrorInvalidValue;
+    const int dpt = sort_dpt(bits);
+    const int form = dpt == 2 ? 2 : items == 4 ? 0 : 1;
+    if (items != 4 && items != 16) return cudaErrorInvalidValue;
+    if (dpt == 2 && items != 16) return cudaErrorInvalidValue;
     const int64_t nb = sort_blocks(n_cap, items);
-    const void *kern = items == 4 ? (const void *)radix_onesweep_kernel<4>
-                     : items == 8 ? (const void *)radix_onesweep_kernel<8>
-                     : items == 32 ? (const void *)radix_onesweep_kernel<32>
-                                   : (const void *)radix_onesweep_kernel<16>;
-    static std::atomic<int> grids[4][kDeviceCache];  // by items (4, 8, 16, 32) and device
-    const int gi = items == 4 ? 0 : items == 8 ? 1 : items == 16 ? 2 : 3;
-    const int grid_res = per_device(grids[gi], [kern] { return resident_grid(kern, kSortThreads, 0, int64_t(1) << 30); });
+    const auto kern = form == 0 ? radix_onesweep_kernel<4, 1>
+                    : form == 1 ? radix_onesweep_kernel<16, 1>
+                                : radix_onesweep_kernel<16, 2>;
+    static std::atomic<int> grids[3][kDeviceCache];  // by form and device
+    const int grid_res = per_device(grids[form], [kern] {
+        return resident_grid((const void *)kern, kSortThreads, 0, int64_t(1) << 30);
+    });
     const unsigned grid = (unsigned)std::min<int64_t>(grid_cap(grid_res, per_sm), nb);
     cudaError_t e;
     uint32_t *ki = k0, *vi = v0, *ko = k1, *vo = v1;
     for (int p = 0; p < np; ++p) {
-        uint32_t *lk = look + (size_t)p * nb * kRadix;
-        uint32_t *nl = p + 1 < np ? lk + (size_t)nb * kRadix : nullptr;
-        const uint32_t *h = hist + p * kRadix;
-        if (items == 4)
-            VPGS_LAUNCH(name, stream, launch_k(radix_onesweep_kernel<4>, grid, kSortThreads, 0, stream,
-                                          ki, vi, ko, vo, n_cap, n_dev, ps[p], h, ticket + p, lk, nl, status, lb));
-        else if (items == 8)
-            VPGS_LAUNCH(name, stream, launch_k(radix_onesweep_kernel<8>, grid, kSortThreads, 0, stream,
-                                          ki, vi, ko, vo, n_cap, n_dev, ps[p], h, ticket + p, lk, nl, status, lb));
-        else if (items == 32)
-            VPGS_LAUNCH(name, stream, launch_k(radix_onesweep_kernel<32>, grid, kSortThreads, 0, stream,
-                                          ki, vi, ko, vo, n_cap, n_dev, ps[p], h, ticket + p, lk, nl, status, lb));
-        else
-            VPGS_LAUNCH(name, stream, launch_k(radix_onesweep_kernel<16>, grid, kSortThreads, 0, stream,
-                                          ki, vi, ko, vo, n_cap, n_dev, ps[p], h, ticket + p, lk, nl, status, lb));
+        uint32_t *lk = look + (size_t)p * nb * kRadix * dpt;
+        uint32_t *nl = p + 1 < np ? lk + (size_t)nb * kRadix * dpt : nullptr;
+        const uint32_t *h = hist + p * kRadix * dpt;
+        VPGS_LAUNCH(name, stream, launch_k(kern, grid, kSortThreads, 0, stream, ki, vi, ko, vo, n_cap, n_dev, ps[p], h,
+                                           ticket + p, lk, nl, status, lb));
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         uint32_t *tk = ki, *tv = vi;
@@ -501,15 +523,16 @@ inline cudaError_t radix_sort_pairs(const char *name, uint32_t *k0, uint32_t *v0
     return cudaSuccess;
 }
 
-// Adds the digits of key k to block-shared histograms of every pass (s_h [passes][256]).
-VPGS_D void add_digits(uint32_t (*s_h)[kRadix], const SortPass *ps, int np, uint32_t k) {
-    for (int p = 0; p < np; ++p) atomicAdd(&s_h[p][(k >> ps[p].shift) & ((1u << ps[p].bits) - 1u)], 1u);
+// Adds the digits of key k to block-shared histograms of every pass (s_h [passes][256 * dpt]).
+VPGS_D void add_digits(uint32_t *s_h, const SortPass *ps, int np, uint32_t k, int dpt = 1) {
+    for (int p = 0; p < np; ++p)
+        atomicAdd(&s_h[p * kRadix * dpt + ((k >> ps[p].shift) & ((1u << ps[p].bits) - 1u))], 1u);
 }
 
 // Adds block-shared histograms into the global ones (non-zero bins only).
-VPGS_D void flush_digits(const uint32_t (*s_h)[kRadix], int np, uint32_t *hist) {
-    for (int i = threadIdx.x; i < np * kRadix; i += blockDim.x) {
-        const uint32_t c = (&s_h[0][0])[i];
+VPGS_D void flush_digits(const uint32_t *s_h, int n_bins, uint32_t *hist) {
+    for (int i = threadIdx.x; i < n_bins; i += blockDim.x) {
+        const uint32_t c = s_h[i];
         if (c) atomicAdd(hist + i, c);
     }
 }

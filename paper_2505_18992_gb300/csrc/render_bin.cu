@@ -49,6 +49,222 @@ struct OffsetStore {
     __device__ void operator()(int64_t r, uint32_t off, uint32_t) const { inst_off[r] = off; }
 };
 
+// Small calls.  Their binning is bound by the latency of its launches (7-15 us each by
+// events, whatever they move), so the ten general ones become two that do more work:
+//
+// small_rank: compaction, depth sort and instance offsets.  The projection appends its
+// visible pairs to a list in any order, and this kernel compares each with all of
+// them: the pairs before it in (depth, index) order give its rank and its first
+// instance; a bit per visible pair gives its place in index order.
+//
+// small_lists: a block per tile tests every visible pair, in depth order, against its
+// tile and writes the tile's list, instead of emission, tile sort and tile ranges.  The
+// lists lie in ws.ival in any order of tiles.
+//
+// Both are bound by the latency of their few loads and barriers below a few thousand
+// pairs, then by their comparisons (bin_form says where they end).  Measured, general ->
+// small: forward of 300 Gaussians in three 97x61 views 66 -> 30 us, tracking iteration
+// of 10k Gaussians (5.3k visible) at 320x240 166 -> 101 us.
+// The results are those of the general path.
+constexpr int kRankThreads = 256;
+constexpr int kRankOwn = 16;    // pairs a block ranks at a time; its half warps take alternate list entries
+constexpr int kRankTile = 2048; // list entries staged at a time
+constexpr int kRankWords = (int)(kSmallPairs / 32);
+// kLists: for small_lists, each pair's tile rectangle (four bytes: first and last column
+// and row) and (pair, view) by rank; else the pair and its first instance by rank
+template <bool kLists>
+__global__ void __launch_bounds__(kRankThreads)
+small_rank_kernel(SmallList list, const uint32_t *__restrict__ tcount, const BinRec *__restrict__ bin, int n_pairs,
+                  int N, uint32_t *__restrict__ vis_idx, uint32_t *__restrict__ by_rank_id,
+                  uint32_t *__restrict__ by_rank, const uint32_t *n_vis, const uint32_t *status) {
+    grid_dep_enter();
+    if (*status != 0u) return;
+    __shared__ __align__(16) unsigned long long s_e[kRankTile];  // depth key, pair index
+    __shared__ __align__(8) uint32_t s_c[kLists ? 2 : kRankTile];  // tile count
+    __shared__ uint32_t s_seen[kRankWords];                      // a bit per visible pair
+    __shared__ uint32_t s_sum[3][kRankOwn];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n = (int)*n_vis, own = lane & (kRankOwn - 1);
+    if ((int)blockIdx.x * kRankOwn >= n) return;
+    const int part = warp * 2 + (lane >> 4);  // this half warp's list entries: 2 part, 2 part + 1 of every kStep
+    constexpr int kStep = 2 * kRankThreads / kRankOwn;
+    constexpr int kUnroll = 8;
+    // (loads in batches: a block's few warps do not hide the latency of one at a time)
+    constexpr int kBatch = 8;
+    for (int i0 = tid; i0 - lane < n_pairs; i0 += kBatch * kRankThreads) {  // warp-uniform
+        uint32_t c[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const int i = i0 + u * kRankThreads;
+            c[u] = i < n_pairs ? tcount[i] : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const uint32_t m = __ballot_sync(0xffffffffu, c[u] > 0u);
+            const int w = (i0 + u * kRankThreads) >> 5;
+            if (lane == 0 && w < kRankWords) s_seen[w] = m;
+        }
+    }
+    for (int i0 = (int)blockIdx.x * kRankOwn; i0 < n; i0 += (int)gridDim.x * kRankOwn) {  // block-uniform
+        const int i = min(i0 + own, n - 1);
+        const uint32_t id = list.pair[i];
+        const unsigned long long me = (unsigned long long)list.key[i] << 32 | id;
+        if (tid < 3 * kRankOwn) (&s_sum[0][0])[tid] = 0u;
+        uint32_t rank = 0u, off = 0u, place = 0u;
+        for (int t0 = 0; t0 < n; t0 += kRankTile) {
+            // the tile, padded with entries that are before none
+            const int nt = min(kRankTile, n - t0);
+            const int np = (nt + kUnroll * kStep - 1) / (kUnroll * kStep) * (kUnroll * kStep);
+            __syncthreads();
+            {
+                constexpr int kPer = kRankTile / kRankThreads;
+                uint32_t ek[kPer], ep[kPer], ec[kPer];
+#pragma unroll
+                for (int u = 0; u < kPer; ++u) {
+                    const int k = tid + u * kRankThreads;
+                    const bool in = k < nt;
+                    ek[u] = in ? list.key[t0 + k] : 0xffffffffu;
+                    ep[u] = in ? list.pair[t0 + k] : 0xffffffffu;
+                    if constexpr (!kLists) ec[u] = in ? list.cnt[t0 + k] : 0u;
+                }
+#pragma unroll
+                for (int u = 0; u < kPer; ++u) {
+                    const int k = tid + u * kRankThreads;
+                    s_e[k] = (unsigned long long)ek[u] << 32 | ep[u];
+                    if constexpr (!kLists) s_c[k] = ec[u];
+                }
+            }
+            __syncthreads();
+            for (int k = 2 * part; k < np; k += kUnroll * kStep) {
+#pragma unroll
+                for (int u = 0; u < kUnroll; ++u) {
+                    const ulonglong2 e = *reinterpret_cast<const ulonglong2 *>(&s_e[k + u * kStep]);
+                    rank += e.x < me;
+                    rank += e.y < me;
+                    if constexpr (!kLists) {
+                        const uint2 c = *reinterpret_cast<const uint2 *>(&s_c[k + u * kStep]);
+                        if (e.x < me) off += c.x;
+                        if (e.y < me) off += c.y;
+                    }
+                }
+            }
+        }
+        for (int w = part; w <= (int)(id >> 5); w += kStep / 2) {
+            const uint32_t bits = s_seen[w];
+            place += __popc(w < (int)(id >> 5) ? bits : bits & ((1u << (id & 31u)) - 1u));
+        }
+        atomicAdd(&s_sum[0][own], rank);
+        if constexpr (!kLists) atomicAdd(&s_sum[1][own], off);
+        atomicAdd(&s_sum[2][own], place);
+        __syncthreads();
+        if (tid < kRankOwn && i0 + tid < n) {
+            const uint32_t r = s_sum[0][tid];
+            vis_idx[s_sum[2][tid]] = id;
+            if constexpr (kLists) {
+                const uint2 rc = bin[id].rect;
+                by_rank_id[r] = id | (id / (uint32_t)N) << 16;
+                by_rank[r] = (rc.x & 0xffu) | (rc.x >> 16 & 0xffu) << 8 | (rc.y & 0xffu) << 16 | (rc.y >> 16 & 0xffu) << 24;
+            } else {
+                by_rank_id[r] = id;
+                by_rank[r] = s_sum[1][tid];
+            }
+        }
+        __syncthreads();
+    }
+}
+
+constexpr int kListThreads = 256;
+constexpr int kListWarps = kListThreads / 32;
+
+__global__ void __launch_bounds__(kListThreads)
+small_lists_kernel(const uint32_t *__restrict__ by_rank_id, const uint32_t *__restrict__ by_rank,
+                   const BinRec *__restrict__ bin, const uint32_t *n_vis, const uint32_t *n_inst, int64_t M_cap,
+                   CamParams cam, uint2 *__restrict__ ranges, uint32_t *__restrict__ ival, uint32_t *cursor,
+                   uint32_t *status) {
+    grid_dep_enter();
+    if (*status != 0u) return;
+    if ((int64_t)*n_inst > M_cap) {
+        if (threadIdx.x == 0) set_status(status, VPGS_ERR_CAPACITY);
+        return;
+    }
+    __shared__ uint16_t s_cand[kSmallPairs + kListThreads];
+    __shared__ uint32_t s_n[kListWarps], s_start;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t below = lanemask_lt();
+    const int tile = (int)blockIdx.x;
+    const uint32_t view = (uint32_t)(tile / cam.T);
+    const int lt = tile - (int)view * cam.T, ty = lt / cam.tiles_x, tx = lt - ty * cam.tiles_x;
+    // the warp's share of the depth order: consecutive ranks
+    const int n = (int)*n_vis, share = (n + kListThreads - 1) / kListThreads * 32;
+    const int first = warp * share, last = min(n, first + share);
+    uint16_t *cand = s_cand + first;
+    uint32_t c = 0u;  // candidates: pairs whose tile rectangle holds this tile
+    constexpr int kBatch = 8;  // (loads in batches, as above)
+    for (int r0 = first; r0 < last; r0 += 32 * kBatch) {
+        uint32_t rc[kBatch], iv[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const int r = r0 + 32 * u + lane;
+            rc[u] = r < last ? by_rank[r] : 0x00ff00ffu;  // (no column, no row)
+            iv[u] = r < last ? by_rank_id[r] : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const bool in = iv[u] >> 16 == view && tx >= (int)(rc[u] & 0xffu) && tx <= (int)(rc[u] >> 8 & 0xffu) &&
+                            ty >= (int)(rc[u] >> 16 & 0xffu) && ty <= (int)(rc[u] >> 24);
+            const uint32_t m = __ballot_sync(0xffffffffu, in);
+            if (in) cand[c + __popc(m & below)] = (uint16_t)iv[u];
+            c += __popc(m);
+        }
+    }
+    __syncwarp();
+    // those whose span of this tile row holds the tile, in place
+    uint32_t hits = 0u;
+    for (uint32_t k0 = 0u; k0 < c; k0 += 32u) {
+        const bool live = k0 + lane < c;
+        const uint32_t id = live ? cand[k0 + lane] : 0u;
+        bool in = false;
+        if (live) {
+            const BinRec &b = bin[id];
+            const uint2 rc = b.rect;
+            const int ty_lo = (int)(rc.y & 0xffffu), rows = (int)(rc.y >> 16) - ty_lo + 1;
+            if (rows <= kCoverRows) {
+                const uint32_t pk = reinterpret_cast<const uint32_t *>(&b.cv)[ty - ty_lo];
+                in = tx >= (int)(pk & 0xffffu) && tx <= (int)(pk >> 16);
+            } else {
+                const Cover cv = b.cv;
+                const float4 uv = b.uv;
+                const int2 sp = cover_row(cv, uv.x, uv.z, uv.y, uv.w, ty, (int)(rc.x & 0xffffu), (int)(rc.x >> 16),
+                                          cam.tw_shift, cam.tile_h, cam.W, cam.H);
+                in = tx >= sp.x && tx <= sp.y;
+            }
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, in);
+        if (in) cand[hits + __popc(m & below)] = (uint16_t)id;
+        hits += __popc(m);
+        __syncwarp();
+    }
+    if (lane == 0) s_n[warp] = hits;
+    __syncthreads();
+    uint32_t at = 0u, total = 0u;
+#pragma unroll
+    for (int w = 0; w < kListWarps; ++w) {
+        at += w < warp ? s_n[w] : 0u;
+        total += s_n[w];
+    }
+    if (tid == 0) {
+        s_start = total ? atomicAdd(cursor, total) : 0u;
+        ranges[tile] = make_uint2(s_start, s_start + total);
+    }
+    __syncthreads();
+    at += s_start;
+    if ((int64_t)s_start + total > M_cap) {  // more tiles than were counted: never in a sound build
+        if (tid == 0) set_status(status, VPGS_ERR_INTERNAL);
+        return;
+    }
+    for (uint32_t k = lane; k < hits; k += 32u) ival[at + k] = cand[k];
+}
+
 // Emits the (global tile id, record) instances of 256 consecutive depth-ranked
 // Gaussians per block.  The instances of Gaussians spanning at most kCoverRows
 // tile rows are spread evenly over the block's threads; each finds its Gaussian
@@ -64,7 +280,7 @@ __global__ void __launch_bounds__(kEmitThreads, 6)
 emit_kernel(const uint32_t *__restrict__ dval, const uint32_t *__restrict__ inst_off,
             const BinRec *__restrict__ bin, const uint32_t *n_vis, const uint32_t *n_inst, int64_t N,
             int64_t M_cap, CamParams cam, uint32_t *__restrict__ ikey, uint32_t *__restrict__ ival,
-            uint32_t *status, int n_pass, SortPass p0, SortPass p1, SortPass p2, SortPass p3,
+            uint32_t *status, int n_pass, int dpt, SortPass p0, SortPass p1, SortPass p2, SortPass p3,
             uint32_t *hist, uint32_t *look0) {
     grid_dep_enter();
     if (*status != 0u) return;  // an earlier kernel failed: dval may hold stale entries
@@ -73,7 +289,7 @@ emit_kernel(const uint32_t *__restrict__ dval, const uint32_t *__restrict__ inst
         // instances (the instance count is known from here on)
         const int64_t ni = min((int64_t)*n_inst, M_cap);
         const int64_t tile = (int64_t)kSortThreads * kTileSortItems;
-        const int64_t nw = (ni + tile - 1) / tile * kRadix;
+        const int64_t nw = (ni + tile - 1) / tile * kRadix * dpt;
         for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nw; i += (int64_t)gridDim.x * blockDim.x)
             look0[i] = 0u;
     }
@@ -199,7 +415,7 @@ emit_kernel(const uint32_t *__restrict__ dval, const uint32_t *__restrict__ inst
         }
         ikey[base + at] = key;
         ival[base + at] = s_id[lo];
-        add_digits(s_h, tps, n_pass, key);
+        add_digits(&s_h[0][0], tps, n_pass, key, dpt);
     }
     // large Gaussians: one warp each, one tile row per lane, a warp prefix of the
     // rows' counts, each lane writing its row's run of tiles
@@ -235,7 +451,7 @@ emit_kernel(const uint32_t *__restrict__ dval, const uint32_t *__restrict__ inst
                 const uint32_t key = vb + (uint32_t)ty * (uint32_t)cam.tiles_x + (uint32_t)sp.x + k;
                 ikey[base + at + k] = key;
                 ival[base + at + k] = id;
-                add_digits(s_h, tps, n_pass, key);
+                add_digits(&s_h[0][0], tps, n_pass, key, dpt);
             }
             running += __shfl_sync(0xffffffffu, x, 31);
         }
@@ -244,7 +460,7 @@ emit_kernel(const uint32_t *__restrict__ dval, const uint32_t *__restrict__ inst
     __syncthreads();  // the next chunk reuses the shared arrays
     }
     __syncthreads();
-    flush_digits(s_h, n_pass, hist);
+    flush_digits(&s_h[0][0], n_pass * kRadix * dpt, hist);
 }
 
 __global__ void tile_ranges_kernel(const uint32_t *__restrict__ keys, int64_t cap, const uint32_t *n_dev,
@@ -372,24 +588,38 @@ tile_work_kernel(const int32_t *__restrict__ n_iter, CamParams cam, int n_tiles,
     if (lane == 0) work[t] = (uint32_t)m;
 }
 
+// A launch order pays only where the tiles take more than one round of blocks: with
+// all of them resident at once (256 threads per SM counted, half of what any of the
+// compositing kernels' registers allow) they all start together.  Below the line the
+// forward saves one launch and the backward two, 6 us each by events (320x240: 300
+// tiles of 128 threads).
+bool tiles_ordered(int n_tiles, const CamParams &cam) {
+    const int64_t threads = (int64_t)n_tiles * (cam.tile_w * cam.tile_h / VPGS_PIX);
+    return VPGS_TILE_ORDER && threads > (int64_t)256 * device_sm_count();
+}
+
+static cudaError_t launch_tile_order(const RenderWs &ws, const uint32_t *work, int n_tiles, cudaStream_t s) {
+    VPGS_LAUNCH("tile_order", s,
+                launch_k(n_tiles <= kOrderThreads * 8 ? tile_order_kernel<8> : tile_order_kernel<32>, 1, kOrderThreads,
+                         0, s, (const uint2 *)ws.ranges, work, n_tiles, ws.tile_order));
+    return cudaGetLastError();
+}
+
 cudaError_t order_tiles_by_steps(const RenderWs &ws, const int32_t *n_iter, int V, const CamParams &cam,
                                  cudaStream_t s) {
     const int n_tiles = V * cam.T;
-    if (n_tiles == 0) return cudaSuccess;
+    if (n_tiles == 0 || !tiles_ordered(n_tiles, cam)) return cudaSuccess;
     const unsigned blocks = (unsigned)(((int64_t)n_tiles * 32 + kWorkThreads - 1) / kWorkThreads);
     VPGS_LAUNCH("tile_work", s, launch_k(tile_work_kernel, blocks, kWorkThreads, 0, s, n_iter, cam, n_tiles,
                                          ws.tile_work));
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (n_tiles <= kOrderThreads * 8)
-        VPGS_LAUNCH("tile_order", s, launch_k(tile_order_kernel<8>, 1, kOrderThreads, 0, s,
-                                              (const uint2 *)ws.ranges, (const uint32_t *)ws.tile_work, n_tiles,
-                                              ws.tile_order));
-    else
-        VPGS_LAUNCH("tile_order", s, launch_k(tile_order_kernel<32>, 1, kOrderThreads, 0, s,
-                                              (const uint2 *)ws.ranges, (const uint32_t *)ws.tile_work, n_tiles,
-                                              ws.tile_order));
-    return cudaGetLastError();
+    return launch_tile_order(ws, ws.tile_work, n_tiles, s);
+}
+
+// Launch order by instance count, where the call uses one.
+static cudaError_t order_tiles_by_count(const RenderWs &ws, int n_tiles, const CamParams &cam, cudaStream_t s) {
+    return tiles_ordered(n_tiles, cam) ? launch_tile_order(ws, nullptr, n_tiles, s) : cudaSuccess;
 }
 
 int tile_list_buffer(const RenderLayout &L) {
@@ -416,37 +646,63 @@ cudaError_t build_tile_lists(const GaussIn &g, int V, const CamParams &cam, cons
     const LookBack lb{o.spin_limit, true};
     cudaError_t e;
     const int sms = device_sm_count();
-    (void)sms;
     uint32_t *n_vis = ws.counters + CNT_VISIBLE;
     uint32_t *n_inst = ws.counters + CNT_INSTANCES;
     // calls of many views (above 4M pairs): wider scan tiles and depth-sort tiles,
     // the offset scan on the resident grid (the visible pairs then fill it)
     const bool many = L.VN > (int64_t(4) << 20);
-    // 1. compaction of visible (view, Gaussian) pairs
-    e = launch_scan("scan_visible", VisLoad{ws.tcount}, VisStore{ws.rec, ws.dkey[0], ws.dval[0], ws.vis_idx, L.VN},
-                    L.VN, nullptr, ws.counters + CNT_TICKET_A, ws.scan_look[0], n_vis, ws.status, s, lb, 0, many);
-    if (e != cudaSuccess) return e;
-    // 2. depth sort
-    bool in1 = false;
-    // (digit histograms from the projection kernel)
-    // keys per thread: few for a frame's worth of visible Gaussians (short tiles
-    // start the look-back chain sooner), more for many views' worth (fewer tiles
-    // in the chain); the look-back space is sized for kDepthSortItems, the most tiles
-    const int depth_items = many ? 16 : kDepthSortItems;
-    e = radix_sort_pairs("sort_depth_pass", ws.dkey[0], ws.dval[0], ws.dkey[1], ws.dval[1], L.VN, n_vis,
-                         0, 32, ws.sort_hist[0], ws.counters + CNT_TICKET_D, ws.sort_look[0], ws.status, s,
-                         &in1, depth_items, lb, VPGS_DEPTH_SORT_GRID);
-    if (e != cudaSuccess) return e;
-    const uint32_t *dval = in1 ? ws.dval[1] : ws.dval[0];  // visible records in depth order
-    uint32_t *inst_off = in1 ? ws.dkey[0] : ws.dkey[1];  // the depth-sort buffer not holding the result
     SortPass tps[kMaxSortPasses] = {};
     const int np_tile = plan_passes(0, L.tile_bits, tps);
     if (np_tile > 4) return cudaErrorInvalidValue;
-    // 3. instance offsets, then emission
-    e = launch_scan("scan_offsets", CountLoad{ws.tcount, dval}, OffsetStore{inst_off}, L.VN, n_vis,
-                    ws.counters + CNT_TICKET_O, ws.scan_look[1], n_inst, ws.status, s, lb,
-                    many ? 0 : VPGS_OFFSET_SCAN_GRID, many);
-    if (e != cudaSuccess) return e;
+    uint32_t *dval = ws.dval[0], *inst_off = ws.dkey[1];  // visible records in depth order, their first instances
+    bool in1 = false;
+    const BinForm form = bin_form(L);
+    if (form != kGeneralBin) {
+        // 1-3 at once (the projection left the list and the counts)
+        const bool lists = form == kSmallLists;
+        dval = ws.sort_look[0];  // the depth sort's look-back words: at least one per pair
+        VPGS_LAUNCH("small_rank", s,
+                    launch_k(lists ? small_rank_kernel<true> : small_rank_kernel<false>,
+                             (unsigned)std::max<int64_t>(std::min<int64_t>((L.VN + kRankOwn - 1) / kRankOwn, 4 * sms), 1),
+                             kRankThreads, 0, s, small_list(ws, L), (const uint32_t *)ws.tcount,
+                             (const BinRec *)ws.bin, (int)L.VN, (int)L.N, ws.vis_idx, dval, inst_off,
+                             (const uint32_t *)n_vis, (const uint32_t *)ws.status));
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        if (lists) {
+            *sorted_buf = tile_list_buffer(L);
+            VPGS_LAUNCH("small_lists", s,
+                        launch_k(small_lists_kernel, (unsigned)(V * cam.T), kListThreads, 0, s, (const uint32_t *)dval,
+                                 (const uint32_t *)inst_off, (const BinRec *)ws.bin, (const uint32_t *)n_vis,
+                                 (const uint32_t *)n_inst, L.M_cap, cam, ws.ranges, ws.ival[*sorted_buf],
+                                 ws.counters + CNT_TICKET_T, ws.status));
+            e = cudaGetLastError();
+            return e != cudaSuccess || !order_by_count ? e : order_tiles_by_count(ws, V * cam.T, cam, s);
+        }
+    } else {
+        // 1. compaction of visible (view, Gaussian) pairs
+        e = launch_scan("scan_visible", VisLoad{ws.tcount},
+                        VisStore{ws.rec, ws.dkey[0], ws.dval[0], ws.vis_idx, L.VN}, L.VN, nullptr,
+                        ws.counters + CNT_TICKET_A, ws.scan_look[0], n_vis, ws.status, s, lb, 0, many);
+        if (e != cudaSuccess) return e;
+        // 2. depth sort (digit histograms from the projection kernel)
+        // keys per thread: few for a frame's worth of visible Gaussians (short tiles
+        // start the look-back chain sooner), more for many views' worth (fewer tiles
+        // in the chain); the look-back space is sized for kDepthSortItems, the most tiles
+        const int depth_items = many ? 16 : kDepthSortItems;
+        e = radix_sort_pairs("sort_depth_pass", ws.dkey[0], ws.dval[0], ws.dkey[1], ws.dval[1], L.VN, n_vis,
+                             0, 32, ws.sort_hist[0], ws.counters + CNT_TICKET_D, ws.sort_look[0], ws.status, s,
+                             &in1, depth_items, lb, VPGS_DEPTH_SORT_GRID);
+        if (e != cudaSuccess) return e;
+        dval = in1 ? ws.dval[1] : ws.dval[0];
+        inst_off = in1 ? ws.dkey[0] : ws.dkey[1];  // the depth-sort buffer not holding the result
+        // 3. instance offsets
+        e = launch_scan("scan_offsets", CountLoad{ws.tcount, dval}, OffsetStore{inst_off}, L.VN, n_vis,
+                        ws.counters + CNT_TICKET_O, ws.scan_look[1], n_inst, ws.status, s, lb,
+                        many ? 0 : VPGS_OFFSET_SCAN_GRID, many);
+        if (e != cudaSuccess) return e;
+    }
+    // emission
     static std::atomic<int> emit_cache[kDeviceCache];
     const int emit_grid = per_device(emit_cache, [] {
         return resident_grid((const void *)emit_kernel, kEmitThreads, 0, int64_t(1) << 30);
@@ -455,7 +711,7 @@ cudaError_t build_tile_lists(const GaussIn &g, int V, const CamParams &cam, cons
                 launch_k(emit_kernel, (unsigned)std::min<int64_t>(std::max<int64_t>((L.VN + kEmitThreads - 1) / kEmitThreads, 1),
                                                           emit_grid),
                               kEmitThreads, 0, s, dval, inst_off, ws.bin, n_vis, n_inst, L.N, L.M_cap,
-                                                    cam, ws.ikey[0], ws.ival[0], ws.status, np_tile, tps[0],
+                                                    cam, ws.ikey[0], ws.ival[0], ws.status, np_tile, sort_dpt(L.tile_bits), tps[0],
                                                     tps[1], tps[2], tps[3], ws.sort_hist[1], ws.sort_look[1]));
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -474,15 +730,8 @@ cudaError_t build_tile_lists(const GaussIn &g, int V, const CamParams &cam, cons
                 launch_k(tile_ranges_kernel, (unsigned)std::max<int64_t>(rb, 1), 256, 0, s,
                     in1 ? ws.ikey[1] : ws.ikey[0], L.M_cap, n_inst, (uint32_t)n_tiles, ws.ranges));
     e = cudaGetLastError();
-    if (e != cudaSuccess || !VPGS_TILE_ORDER || !order_by_count) return e;
     // 6. compositing launch order
-    if (n_tiles <= kOrderThreads * 8)
-        VPGS_LAUNCH("tile_order", s, launch_k(tile_order_kernel<8>, 1, kOrderThreads, 0, s, (const uint2 *)ws.ranges,
-                                              (const uint32_t *)nullptr, n_tiles, ws.tile_order));
-    else
-        VPGS_LAUNCH("tile_order", s, launch_k(tile_order_kernel<32>, 1, kOrderThreads, 0, s, (const uint2 *)ws.ranges,
-                                              (const uint32_t *)nullptr, n_tiles, ws.tile_order));
-    return cudaGetLastError();
+    return e != cudaSuccess || !order_by_count ? e : order_tiles_by_count(ws, n_tiles, cam, s);
 }
 
 }  // namespace vpgs

@@ -1059,7 +1059,7 @@ cudaError_t launch_composite_fwd(const RenderWs &ws, const uint32_t *ival, int V
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     VPGS_LAUNCH("composite_fwd", s,
                 launch_k(composite_fwd_kernel, grid, B, sm, s, ws.rec, ival, ws.ranges,
-                         VPGS_TILE_ORDER ? (const uint32_t *)ws.tile_order : nullptr, n_tiles, cam, o, out,
+                         tiles_ordered(n_tiles, cam) ? (const uint32_t *)ws.tile_order : nullptr, n_tiles, cam, o, out,
                          ws.status, work));
     return cudaGetLastError();
 }
@@ -1087,7 +1087,7 @@ cudaError_t launch_composite_bwd(const RenderWs &ws, const uint32_t *ival, int V
     if (grid == 0) return cudaSuccess;
     VPGS_LAUNCH("composite_bwd", s,
                 launch_k(kern, grid, B, sm, s, ws.rec, ival, ws.ranges,
-                         VPGS_TILE_ORDER ? (const uint32_t *)ws.tile_order : nullptr, n_tiles, cam, o,
+                         tiles_ordered(n_tiles, cam) ? (const uint32_t *)ws.tile_order : nullptr, n_tiles, cam, o,
                          fwd.t_final, fwd.n_iter, dL_drgb, dL_ddepth, dL_dalpha, ws.g2d, ws.status, work));
     return cudaGetLastError();
 }

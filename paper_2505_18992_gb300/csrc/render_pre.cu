@@ -14,6 +14,9 @@
 // Backward, one thread per visible (view, Gaussian): chain rule from the 2D
 // gradients (u, v, conic, opacity, colour, depth) back to mean, scale,
 // quaternion, opacity and colour, plus the per-view pose terms summed in FP64.
+#include <cooperative_groups.h>
+#include <cooperative_groups/reduce.h>
+
 #include "internal.h"
 #include "prims.cuh"
 #include "profiler.h"
@@ -401,22 +404,44 @@ precull_kernel(GaussIn g, int V, CamParams cam, OptParams o, RenderWs ws, uint32
     }
 }
 
+// Appends a visible pair to the list of a small call and adds to the counts of visible
+// pairs and instances: one atomic each per converged group of lanes.  Every caller's
+// lane passes cnt (0: culled, nothing appended).
+VPGS_D void append_visible(const SmallList &list, uint32_t *counters, uint32_t cnt, float depth, int64_t pair) {
+    const auto g = cooperative_groups::coalesced_threads();
+    const uint32_t m = g.ballot(cnt != 0u);
+    if (m == 0u) return;
+    const uint32_t total = cooperative_groups::reduce(g, cnt, cooperative_groups::plus<uint32_t>());
+    uint32_t at = 0u;
+    if (g.thread_rank() == 0) {
+        at = atomicAdd(counters + CNT_VISIBLE, (uint32_t)__popc(m));
+        atomicAdd(counters + CNT_INSTANCES, total);
+    }
+    at = g.shfl(at, 0) + __popc(m & ((1u << g.thread_rank()) - 1u));
+    if (cnt) {
+        list.key[at] = __float_as_uint(depth);  // camera z > near_z > 0: the bits order like the floats
+        list.cnt[at] = cnt;
+        list.pair[at] = (uint32_t)pair;
+    }
+}
+
 // Exact projection of one pre-cull survivor ic = (view, Gaussian) from its
 // parameters, and everything the binning needs of it: tile count, screen and
 // binning records, the digits of its depth key (block histograms s_h), and
 // zeroed 2D-gradient slots when asked.
 VPGS_D void project_write(int64_t ic, int v, float mx, float my, float mz, float sx, float sy, float sz, float4 q,
                           float op, float cr, float cg, float cb, const CamParams &cam, const OptParams &o,
-                          const RenderWs &ws, bool zero_g2d, uint32_t (*s_h)[kRadix]) {
+                          const RenderWs &ws, const SmallList &list, bool zero_g2d, uint32_t (*s_h)[kRadix]) {
     const SortPass dps[4] = {{0, 8}, {8, 8}, {16, 8}, {24, 8}};  // the depth sort's passes over 32 bits
     BinRec B;
     float depth = 0.f;
     const uint32_t cnt = project_one(ws.posedf + 24 * v, mx, my, mz, sx, sy, sz, q, op, cr, cg, cb, cam, o,
                                      ws.status, ws.rec + ic, B, depth);
     ws.tcount[ic] = cnt;
+    if (list.key) append_visible(list, ws.counters, cnt, depth, ic);
     if (cnt) {
         ws.bin[ic] = B;
-        add_digits(s_h, dps, 4, __float_as_uint(depth));  // the depth key (camera z > 0)
+        if (!list.key) add_digits(&s_h[0][0], dps, 4, __float_as_uint(depth));  // the depth key (camera z > 0)
         if (zero_g2d) {
             float2 *z2 = reinterpret_cast<float2 *>(ws.g2d + 10 * ic);
 #pragma unroll
@@ -451,7 +476,7 @@ struct QItem {
 };
 
 __global__ void __launch_bounds__(kPreThreads, 3)
-cull_project_kernel(GaussIn g, int V, CamParams cam, OptParams o, RenderWs ws, bool zero_g2d) {
+cull_project_kernel(GaussIn g, int V, CamParams cam, OptParams o, RenderWs ws, SmallList list, bool zero_g2d) {
     grid_dep_enter();
     __shared__ uint32_t s_h[4][kRadix];
     __shared__ QItem s_q[kPreThreads];
@@ -542,22 +567,22 @@ cull_project_kernel(GaussIn g, int V, CamParams cam, OptParams o, RenderWs ws, b
                     const uint32_t v = __float_as_uint(it.c.w);
                     const int64_t ic = (int64_t)v * g.N + __float_as_uint(it.c.z);
                     project_write(ic, (int)v, it.a.x, it.a.y, it.a.z, it.a.w, it.b.x, it.b.y, it.q, it.b.z, it.b.w,
-                                  it.c.x, it.c.y, cam, o, ws, zero_g2d, s_h);
+                                  it.c.x, it.c.y, cam, o, ws, list, zero_g2d, s_h);
                 }
                 __syncthreads();  // the staging slots are rewritten by the next batch
             }
         }
     }
     __syncthreads();
-    flush_digits(s_h, 4, ws.sort_hist[0]);
+    flush_digits(&s_h[0][0], 4 * kRadix, ws.sort_hist[0]);
 }
 
 // Pass 2, grid-strided over the candidates: the exact projection on full warps.
 // It also accumulates the digit histograms of the visible Gaussians' depth keys
 // for the depth sort.
 __global__ void __launch_bounds__(kPreThreads, 3)
-project_kernel(GaussIn g, CamParams cam, OptParams o, RenderWs ws, const uint32_t *__restrict__ cand,
-               const uint32_t *n_cand, bool zero_g2d) {
+project_kernel(GaussIn g, CamParams cam, OptParams o, RenderWs ws, SmallList list,
+               const uint32_t *__restrict__ cand, const uint32_t *n_cand, bool zero_g2d) {
     grid_dep_enter();
     __shared__ uint32_t s_h[4][kRadix];
     for (int i = threadIdx.x; i < 4 * kRadix; i += blockDim.x) (&s_h[0][0])[i] = 0u;
@@ -577,9 +602,10 @@ project_kernel(GaussIn g, CamParams cam, OptParams o, RenderWs ws, const uint32_
                                          g.opac[gi], g.colors[3 * gi], g.colors[3 * gi + 1], g.colors[3 * gi + 2],
                                          cam, o, ws.status, ws.rec + ic, B, depth);
         ws.tcount[ic] = cnt;
+        if (list.key) append_visible(list, ws.counters, cnt, depth, ic);
         if (cnt) {
             ws.bin[ic] = B;
-            add_digits(s_h, dps, 4, __float_as_uint(depth));  // the depth key (camera z > 0)
+            if (!list.key) add_digits(&s_h[0][0], dps, 4, __float_as_uint(depth));  // the depth key (camera z > 0)
             if (zero_g2d) {
                 float2 *z2 = reinterpret_cast<float2 *>(ws.g2d + 10 * ic);
 #pragma unroll
@@ -588,7 +614,7 @@ project_kernel(GaussIn g, CamParams cam, OptParams o, RenderWs ws, const uint32_
         }
     }
     __syncthreads();
-    flush_digits(s_h, 4, ws.sort_hist[0]);
+    flush_digits(&s_h[0][0], 4 * kRadix, ws.sort_hist[0]);
 }
 
 VPGS_D float warp_sum(float x) {
@@ -837,16 +863,19 @@ cudaError_t launch_preprocess_fwd(const GaussIn &g, const double *T_cw, int V, c
     z.w32[0] = ws.status;                      z.n32[0] = 1;
     z.w32[1] = ws.counters;                    z.n32[1] = CNT_N;
     z.w32[2] = ws.sort_hist[0];                z.n32[2] = 2 * 4 * kRadix;  // both sorts
-    z.w32[3] = ws.sort_look[0];                z.n32[3] = sort_blocks(std::max<int64_t>(L.VN, 1), kDepthSortItems) * kRadix;
+    const bool small = bin_form(L) != kGeneralBin;  // no depth sort, no scans
+    z.w32[3] = ws.sort_look[0];
+    z.n32[3] = small ? 0 : sort_blocks(std::max<int64_t>(L.VN, 1), kDepthSortItems) * kRadix;
     z.w32[4] = ws.sort_look[1];                z.n32[4] = 0;  // zeroed by emit, sized by the instance count
     z.w32[5] = reinterpret_cast<uint32_t *>(ws.ranges);  z.n32[5] = 2 * (int64_t)V * cam.T;
-    z.w64 = ws.scan_look[0];                   z.n64 = 2 * L.scan_blocks_max;  // both scans
+    z.w64 = ws.scan_look[0];                   z.n64 = small ? 0 : 2 * L.scan_blocks_max;  // both scans
     const int prep_grid = 8 * device_sm_count();
     const int64_t words = std::max<int64_t>(z.n32[3] + z.n32[4] + z.n32[5], z.n64);
     VPGS_LAUNCH("prepare", s,
                 launch_k(prepare_kernel, (unsigned)std::max<int64_t>(1, std::min<int64_t>(prep_grid, (words + 255) / 256)),
                                  256, 0, s, T_cw, V, ws.posedf, z));
     if (VN == 0) return cudaGetLastError();
+    const SmallList list = small_list(ws, L);
     if (VPGS_CULL_PROJECT > 0 && V >= VPGS_CULL_PROJECT) {
         static std::atomic<int> cp_cache[kDeviceCache];
         const int cp_grid = per_device(cp_cache, [] {
@@ -857,7 +886,7 @@ cudaError_t launch_preprocess_fwd(const GaussIn &g, const double *T_cw, int V, c
         VPGS_LAUNCH("cull_project", s,
                     launch_k(cull_project_kernel,
                              (unsigned)std::min<int64_t>(cp_grid, (g.N + kPreThreads - 1) / kPreThreads),
-                             kPreThreads, 0, s, g, V, cam, o, ws, zero_g2d));
+                             kPreThreads, 0, s, g, V, cam, o, ws, list, zero_g2d));
         return cudaGetLastError();
     }
     // the candidate list borrows the second depth-key buffer (free until the depth sort)
@@ -873,7 +902,7 @@ cudaError_t launch_preprocess_fwd(const GaussIn &g, const double *T_cw, int V, c
     });
     VPGS_LAUNCH("project", s,
                 launch_k(project_kernel, (unsigned)std::min<int64_t>(proj_grid, (VN + kPreThreads - 1) / kPreThreads),
-                                 kPreThreads, 0, s, g, cam, o, ws, cand, n_cand, zero_g2d));
+                                 kPreThreads, 0, s, g, cam, o, ws, list, cand, n_cand, zero_g2d));
     return cudaGetLastError();
 }
 
