@@ -22,10 +22,9 @@
 // carries that scalar instead of B.
 // Per-Gaussian 2D gradient sums of a warp are taken in the Gaussian's whitened frame
 // t = W d: sum dpow t1, sum dpow t2, sum dpow t1^2, sum dpow t1 t2, sum dpow t2^2;
-// then opacity, rgb, z.  Two kernels: the full backward collects its pixels' terms in
-// shared memory and sums them one entry per lane (composite_bwd_kernel); pose
-// tracking sums six of the ten by shuffles (composite_geo_kernel).  Each adds its
-// sums with one atomic per value and warp.
+// then opacity, rgb, z.  The full backward collects its pixels' terms in shared memory
+// and sums them one entry per lane; the geometric one (pose tracking) sums six of the
+// ten by shuffles.  Each adds its sums with one atomic per value and warp.
 // Near-degenerate records (negative y half extent) take the double-float pair
 // evaluation (eval_pair_fine): one warp-uniform branch per list entry.
 #include <type_traits>
@@ -59,6 +58,10 @@ constexpr int kFwdBatch = VPGS_FWD_BATCH;
 #define VPGS_BWD_BATCH 1  // records each thread of the full backward stages per batch (2: 20 KB more, 292 us)
 #endif
 constexpr int kBwdBatch = VPGS_BWD_BATCH;
+#ifndef VPGS_GEO_BATCH
+#define VPGS_GEO_BATCH 2  // the same of the geometric backward (1: 310 us, 2: 288 us)
+#endif
+constexpr int kGeoBatch = VPGS_GEO_BATCH;
 // list entries whose alphas the forward evaluates before blending them (see VPGS_FWD_MAXREG)
 #ifndef VPGS_FWD_WALK
 #define VPGS_FWD_WALK 8
@@ -100,43 +103,15 @@ VPGS_D bool reaches_box(const float4 &a, const float4 &b, float x0, float x1, fl
     return !(m > fmaf(1e-3f, fabsf(level), level) + 1e-3f);
 }
 
-// Compacts the batch positions [0, n) whose Gaussian reaches the warp's pixel
-// rows into list, in ascending order; returns how many (warp-uniform).  A
-// Gaussian is listed when its widened y extent reaches the rows and, for a plain
-// record, its alpha_min ellipse also meets the rows' pixel centres within the
-// tile's columns [0.5, xmax].  All 32 lanes take part.  `fine` tells
-// (warp-uniform) whether a listed record is near-degenerate.
-VPGS_D int warp_list(const float4 *s0, const float4 *s1, int n, float2 band, uint16_t *list, int lane,
-                     bool &fine, float xmax, float lg_amin) {
-    const uint32_t below = (1u << lane) - 1u;
-    int cnt = 0;
-    bool any = false;
-    for (int c0 = 0; c0 < n; c0 += 32) {
-        const int k = c0 + lane;
-        bool touch = false, f = false;
-        if (k < n) {
-            const float4 a = s0[k], b = s1[k];
-            const float ry = b.w;
-            touch = fabsf(a.y - band.x) <= fabsf(ry) + band.y;
-            f = touch && ry < 0.f;
-            if (touch && !f) touch = reaches_box(a, b, 0.5f, xmax, band.x - band.y, band.x + band.y, lg_amin);
-        }
-        const uint32_t m = __ballot_sync(0xffffffffu, touch);
-        any |= __any_sync(0xffffffffu, f);
-        if (touch) list[cnt + __popc(m & below)] = (uint16_t)k;
-        cnt += __popc(m);
-    }
-    __syncwarp();
-    fine = any;
-    return cnt;
-}
-
-// The same list for the packed walks of the forward and the full backward: the byte
-// offsets of the staged records (kRecStage float4 each), first record first or, with
-// kBack, last record first.  kExact (the backward): the ellipse test too.  Without it
-// (the forward) a Gaussian is listed by its y extent alone: both list every Gaussian
-// that blends into a pixel of the rows, so they may differ in what they skip but not
-// in what they blend.
+// Compacts the batch positions [0, n) whose Gaussian reaches the warp's pixel rows
+// into list, as byte offsets of the staged records (kRecStage float4 each), first
+// record first or, with kBack, last record first; returns how many (warp-uniform).  A
+// Gaussian is listed when its widened y extent reaches the rows and, with kExact (the
+// backward) and a plain record, its alpha_min ellipse also meets the rows' pixel
+// centres within the tile's columns [0.5, xmax].  Both forms list every Gaussian that
+// blends into a pixel of the rows, so they may differ in what they skip but not in
+// what they blend.  All 32 lanes take part.  `fine` tells (warp-uniform) whether a
+// listed record is near-degenerate.
 constexpr int kRecStage = 5;  // float4 per staged record: an odd number keeps 16-byte reads by lane conflict-free
 template <bool kExact, bool kBack>
 VPGS_D int warp_offsets(const float4 *s_rec, int n, float2 band, uint16_t *list, int lane, bool &fine, float xmax,
@@ -516,180 +491,6 @@ VPGS_D bool pair_grad(PixState &p, int jj, const PairEval &e, const float4 &b, c
 }
 
 // ---------------------------------------------------------------------------
-// Geometric backward (pose tracking: no opacity or colour gradient is asked): the
-// six sums that the means, covariances, depths and the pose need.  One lane per
-// column pair of pixels, branching pair code and a six-value shuffle reduction per
-// entry.  The two-phase form of the full backward took 250 us instead of 345 us here
-// (1M-Gaussian room, 1200x680), but it adds a warp's terms in another order, and a
-// tracking run feeds on its own roundings: the signs of the L1 loss near its minimum
-// amplify them to pose differences beyond those between two runs of this form.
-// ---------------------------------------------------------------------------
-#ifndef VPGS_GEO_BATCH
-#define VPGS_GEO_BATCH 2  // records each thread stages per batch
-#endif
-constexpr int kGeoBatch = VPGS_GEO_BATCH;
-#ifndef VPGS_BWD_DIRECT
-#define VPGS_BWD_DIRECT 2
-#endif
-constexpr int kDirect = VPGS_BWD_DIRECT;  // at most this many active lanes: per-lane atomics, no reduction
-// register cap (0: only the 512-thread launch bound).  72 registers keep 7 blocks of
-// 4 warps resident per SM: registers are granted in units of 8 per thread, so 73-80
-// would leave room for 6 blocks.  The kernel needs no spill under this cap.
-#ifndef VPGS_GEO_MAXREG
-#define VPGS_GEO_MAXREG 72
-#endif
-#if VPGS_GEO_MAXREG > 0
-#define VPGS_GEO_BOUNDS __maxnreg__(VPGS_GEO_MAXREG)
-#else
-#define VPGS_GEO_BOUNDS __launch_bounds__(kMaxThreads)
-#endif
-
-__global__ void VPGS_GEO_BOUNDS
-composite_geo_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ ival,
-                     const uint2 *__restrict__ ranges, const uint32_t *__restrict__ order, int n_tiles,
-                     CamParams cam, OptParams o,
-                     const float *__restrict__ t_final, const int32_t *__restrict__ n_iter,
-                     const float *__restrict__ dL_drgb, const float *__restrict__ dL_ddepth,
-                     const float *__restrict__ dL_dalpha, float *__restrict__ g2d,
-                     const uint32_t *status, uint32_t *work) {
-    grid_dep_enter();
-    extern __shared__ float4 smem[];
-    const int NT = blockDim.x * kGeoBatch;  // records per batch
-    float4 *s0 = smem, *s1 = smem + NT, *s2 = smem + 2 * NT;
-    uint32_t *s_id = reinterpret_cast<uint32_t *>(smem + 3 * NT);
-    uint16_t *s_wl = reinterpret_cast<uint16_t *>(s_id + NT);             // [NW][NT] per-warp lists
-    __shared__ int s_tile;
-    __shared__ int s_max;
-    if (*status != 0u) return;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int lx = tid % cam.tile_w, ly = tid / cam.tile_w;
-    const float pxl = (float)lx + 0.5f;
-    float pyl[kPix];
-#pragma unroll
-    for (int q = 0; q < kPix; ++q) pyl[q] = (float)(kPix * ly + q) + 0.5f;
-    const float2 band = warp_rows(pyl);
-    const float lg_amin = __log2f(o.alpha_min);
-    uint16_t *wl = s_wl + (size_t)warp * NT;
-    constexpr int NV = 6;
-    const int rs = red_slot<NV>(lane);
-    const int slot = rs >= 0 ? g2d_slot<NV>(rs) : -1;
-    int t = blockIdx.x;
-    for (;;) {
-        if (work) {
-            if (tid == 0) s_tile = (int)atomicAdd(work, 1u);
-            __syncthreads();
-            t = s_tile;
-        }
-        if (tid == 0) s_max = 0;
-        __syncthreads();
-        if (t >= n_tiles) return;
-        const int tile = order ? (int)order[t] : t;  // launch order -> global tile id
-        const TileCoord tc = tile_coord(tile, cam);
-        const int px = tc.tx * cam.tile_w + lx;
-        const float ox = (float)(tc.tx * cam.tile_w), oy = (float)(tc.ty * cam.tile_h);
-        const float xmax = fminf((float)cam.tile_w, (float)cam.W - ox) - 0.5f;  // last pixel centre column
-        const uint2 rg = ranges[tile];
-        const int start = (int)rg.x;
-        const int64_t HW = (int64_t)cam.H * cam.W;
-        PixState ps[kPix];
-        int my_max = 0;
-#pragma unroll
-        for (int q = 0; q < kPix; ++q) {
-            PixState &p = ps[q];
-            p.T = 1.f; p.gC0 = p.gC1 = p.gC2 = p.gD = 0.f; p.last = 0;
-            float gA = 0.f;
-            const int py = tc.ty * cam.tile_h + kPix * ly + q;
-            if (px < cam.W && py < cam.H) {
-                const int64_t pix = (int64_t)tc.v * HW + (int64_t)py * cam.W + px;
-                p.T = t_final[pix];
-                p.last = n_iter[pix];
-                if (dL_drgb) {
-                    const float *gp = dL_drgb + (int64_t)tc.v * 3 * HW + (int64_t)py * cam.W + px;
-                    p.gC0 = gp[0]; p.gC1 = gp[HW]; p.gC2 = gp[2 * HW];
-                }
-                if (dL_ddepth) p.gD = dL_ddepth[pix];
-                if (dL_dalpha) gA = dL_dalpha[pix];
-            }
-            p.gAT = gA * p.T;  // p.T holds T_final here
-            p.beta = fmaf(p.gC0, o.bg0, fmaf(p.gC1, o.bg1, p.gC2 * o.bg2));  // B starts at the background
-            my_max = max(my_max, p.last);
-        }
-        // the warp's own list length: warps whose pixels stop early skip the tail
-        const int warp_max = (int)__reduce_max_sync(0xffffffffu, (unsigned)my_max);
-        if (lane == 0 && warp_max > 0) atomicMax(&s_max, warp_max);
-        __syncthreads();
-        const int list_end = start + min(s_max, (int)rg.y - start);  // n_iter never exceeds the list
-        for (int b1 = list_end; b1 > start; b1 -= NT) {
-            const int b0 = max(start, b1 - NT);
-            const int nb = b1 - b0;
-            __syncthreads();
-#pragma unroll 1
-            for (int u = 0; u < kGeoBatch; ++u) {
-                const int k = tid + u * (int)blockDim.x;
-                if (b0 + k < b1) {
-                    const uint32_t id = ival[b0 + k];
-                    stage(rec[id], ox, oy, s0[k], s1[k], s2[k]);
-                    s_id[k] = id;
-                }
-            }
-            __syncthreads();
-            const int k_end = min(nb, warp_max - (b0 - start));  // warp-uniform
-            bool any_fine;
-            const int nl = warp_list(s0, s1, k_end, band, wl, lane, any_fine, xmax, lg_amin);
-            // back to front; a batch with a near-degenerate record takes the walk that
-            // chooses the precision form per entry (a warp-uniform branch), the others
-            // the plain one
-            auto walk = [&](auto maybe_fine) {
-            for (int i = nl - 1; i >= 0; --i) {
-                const int kk = wl[i];
-                const float4 a = s0[kk], b = s1[kk], c = s2[kk];
-                float v[NV];
-#pragma unroll
-                for (int q = 0; q < NV; ++q) v[q] = 0.f;
-                const int jj = b0 + kk - start;
-                // this thread's pixels against the Gaussian
-                auto grads = [&](auto fine) -> bool {
-                    constexpr bool kFine = decltype(fine)::value;
-                    float4 f;
-                    if constexpr (kFine) f = fine_extra(rec[s_id[kk]], ox, oy, a.x, a.y);
-                    const float2 t0 = kFine ? make_float2(0.f, 0.f) : first_row(pxl, pyl[0], a, b);
-                    bool any = false;
-#pragma unroll
-                    for (int q = 0; q < kPix; ++q) {
-                        const PairEval e = eval_staged<kFine>(q, t0.x, t0.y, pxl, pyl[q], a, b, f, o.alpha_max);
-                        any |= pair_grad(ps[q], jj, e, b, c, o, v);
-                    }
-                    return any;
-                };
-                bool act;
-                if constexpr (decltype(maybe_fine)::value)
-                    act = b.w < 0.f ? grads(std::true_type{}) : grads(std::false_type{});
-                else
-                    act = grads(std::false_type{});
-                const uint32_t am = __ballot_sync(0xffffffffu, act);
-                if (am != 0u && __popc(am) <= kDirect) {
-                    // few active lanes: their own atomics beat a reduction
-                    if (act) {
-                        float *dst = g2d + 10 * (int64_t)s_id[kk];
-#pragma unroll
-                        for (int q = 0; q < NV; ++q)
-                            if (v[q] != 0.f) atomicAdd(dst + g2d_slot<NV>(q), v[q]);
-                    }
-                } else if (am != 0u) {
-                    warp_reduce(v, lane);
-                    if (slot >= 0 && v[0] != 0.f) atomicAdd(g2d + 10 * (int64_t)s_id[kk] + slot, v[0]);
-                }
-            }
-            };
-            if (any_fine) walk(std::true_type{});
-            else walk(std::false_type{});
-        }
-        if (!work) return;
-        __syncthreads();
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Backward.  The ten 2D gradient sums of a Gaussian are linear in two numbers per
 // pixel, its blend weight w and dpow (the gradient of the exponent):
 //   sum w (g_r, g_g, g_b, g_z)   and   sum dpow (1, t1, t2, t1^2, t1 t2, t2^2)
@@ -713,11 +514,26 @@ composite_geo_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
 // kSlots 16 halves the transpose steps but takes 16 KB more per block: 322 us (room).
 // The shuffle form remains for the batches that hold a near-degenerate record, and for
 // pixels or records whose magnitudes could turn 0 * x into a NaN (kOdd).
+//
+// The geometric form (NV = 6: no opacity or colour gradient is asked, as in pose
+// tracking) takes phase 1 without branches but sums each entry by shuffles, in the
+// order and with the roundings it always had: 345 -> 288 us (room), 39 -> 29 us (10k
+// Gaussians at 320x240).  Its two-phase form took 250 us (room), but adds a warp's terms
+// in another order, and a tracking run feeds on its own roundings: the signs of the L1
+// loss near its minimum amplify them to pose differences beyond those between two runs.
 // ---------------------------------------------------------------------------
 #ifndef VPGS_BWD_SLOTS
 #define VPGS_BWD_SLOTS 8
 #endif
 constexpr int kSlots = VPGS_BWD_SLOTS;
+#ifndef VPGS_GEO_WALK
+#define VPGS_GEO_WALK 2
+#endif
+constexpr int kGeoWalk = VPGS_GEO_WALK;  // entries whose alphas the geometric form evaluates at a time
+#ifndef VPGS_BWD_DIRECT
+#define VPGS_BWD_DIRECT 2
+#endif
+constexpr int kDirect = VPGS_BWD_DIRECT;  // at most this many active lanes: per-lane atomics, no reduction
 #ifndef VPGS_BWD_UNROLL
 #define VPGS_BWD_UNROLL 2
 #endif
@@ -742,6 +558,7 @@ static_assert(kPix == 2, "the packed forms hold two rows per lane");
 #define VPGS_BWD_BOUNDS __launch_bounds__(kMaxThreads)
 #endif
 
+template <int NV>
 __global__ void VPGS_BWD_BOUNDS
 composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ ival,
                      const uint2 *__restrict__ ranges, const uint32_t *__restrict__ order, int n_tiles,
@@ -751,16 +568,18 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                      const float *__restrict__ dL_dalpha, float *__restrict__ g2d,
                      const uint32_t *status, uint32_t *work) {
     grid_dep_enter();
-    constexpr int NV = 10;
+    constexpr bool kGeo = NV == 6;
+    constexpr int kTerm = kGeo ? 0 : kSlots * kTermStride, kPixN = kGeo ? 0 : kPixSize;  // float4 per warp
     extern __shared__ float4 smem[];
-    const int NT = blockDim.x * kBwdBatch;  // records per batch
+    constexpr int kBatch = NV == 6 ? kGeoBatch : kBwdBatch;
+    const int NT = blockDim.x * kBatch;  // records per batch
     const int NW = blockDim.x >> 5;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // records: s0, s1 as in the forward, the colour and depth doubled (r, r, g, g), (b, b, z, z), the id
     float4 *s_rec = smem;
-    float4 *s_term = smem + kRecStage * NT + warp * (kSlots * kTermStride);           // this warp's (w, w, dpow, dpow)
-    float4 *s_pix = smem + kRecStage * NT + NW * (kSlots * kTermStride) + warp * kPixSize;  // this warp's -g
-    uint16_t *wl = reinterpret_cast<uint16_t *>(smem + kRecStage * NT + NW * (kSlots * kTermStride + kPixSize)) +
+    float4 *s_term = smem + kRecStage * NT + warp * kTerm;              // this warp's (w, w, dpow, dpow)
+    float4 *s_pix = smem + kRecStage * NT + NW * kTerm + warp * kPixN;  // this warp's -g
+    uint16_t *wl = reinterpret_cast<uint16_t *>(smem + kRecStage * NT + NW * (kTerm + kPixN)) +
                    (size_t)warp * NT;  // this warp's list
     __shared__ int s_tile;
     __shared__ int s_max;
@@ -774,6 +593,23 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
     const float2 band = warp_rows(pyl);
     const float lg_amin = __log2f(o.alpha_min);
     const f2 one2 = pack2(1.f, 1.f);
+    // adds the lanes' values of one entry to its slots: by a shuffle reduction, or where
+    // few lanes blended by their own atomics
+    const int red = red_slot<NV>(lane), slot = red >= 0 ? g2d_slot<NV>(red) : -1;
+    auto add_sums = [&](uint32_t id, float (&v)[NV], bool act) {
+        const uint32_t am = __ballot_sync(0xffffffffu, act);
+        float *dst = g2d + 10 * (int64_t)id;
+        if (am != 0u && __popc(am) <= kDirect) {
+            if (act) {
+#pragma unroll
+                for (int q = 0; q < NV; ++q)
+                    if (v[q] != 0.f) atomicAdd(dst + g2d_slot<NV>(q), v[q]);
+            }
+        } else if (am != 0u) {
+            warp_reduce(v, lane);
+            if (slot >= 0 && v[0] != 0.f) atomicAdd(dst + slot, v[0]);
+        }
+    };
     int t = blockIdx.x;
     for (;;) {
         if (work) {
@@ -828,8 +664,10 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
             my_max = max(my_max, last[q]);
         }
         const bool warp_odd = __any_sync(0xffffffffu, odd);
-        s_pix[2 * lane + lane / kSlots] = make_float4(ng0[0], ng0[1], ng1[0], ng1[1]);
-        s_pix[2 * lane + lane / kSlots + 1] = make_float4(ng2[0], ng2[1], ngd[0], ngd[1]);
+        if constexpr (!kGeo) {
+            s_pix[2 * lane + lane / kSlots] = make_float4(ng0[0], ng0[1], ng1[0], ng1[1]);
+            s_pix[2 * lane + lane / kSlots + 1] = make_float4(ng2[0], ng2[1], ngd[0], ngd[1]);
+        }
         f2 T2 = pack2(T[0], T[1]), beta2 = pack2(beta[0], beta[1]);
         const f2 ng02 = pack2(ng0[0], ng0[1]), ng12 = pack2(ng1[0], ng1[1]), ng22 = pack2(ng2[0], ng2[1]),
                  ngd2 = pack2(ngd[0], ngd[1]), ngat2 = pack2(ngat[0], ngat[1]);
@@ -843,7 +681,7 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
             const int nb = b1 - b0;
             __syncthreads();
 #pragma unroll 1
-            for (int u = 0; u < kBwdBatch; ++u) {
+            for (int u = 0; u < kBatch; ++u) {
                 const int k = tid + u * (int)blockDim.x;
                 if (b0 + k < b1) {
                     const uint32_t id = ival[b0 + k];
@@ -878,7 +716,6 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                     p.gD = -(q ? hi2(ngd2) : lo2(ngd2));
                     p.last = last[q];
                 }
-                const int slot = red_slot<NV>(lane);
                 for (int i = 0; i < nl; ++i) {
                     const float4 *r = rec_at(s_rec, wl[i]);
                     const int kk = wl[i] / (kRecStage * 16);
@@ -902,46 +739,81 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                         return any;
                     };
                     const bool act = b.w < 0.f ? grads(std::true_type{}) : grads(std::false_type{});
-                    if (__any_sync(0xffffffffu, act)) {
-                        warp_reduce(v, lane);
-                        if (slot >= 0 && v[0] != 0.f) atomicAdd(g2d + 10 * (int64_t)id + slot, v[0]);
-                    }
+                    add_sums(id, v, act);
                 }
                 T2 = pack2(ps[0].T, ps[1].T);
                 beta2 = pack2(ps[0].beta, ps[1].beta);
                 continue;
             }
             const int l0 = (last[0] - base) * (kRecStage * 16), l1 = (last[1] - base) * (kRecStage * 16);
+            // (blend weight, negated; dpow) of the lane's pixels for the record at off, zero
+            // where a pixel does not blend; updates T and beta.  t12, t22: the whitened
+            // coordinates of the two rows.  na: the negated alphas, masked; r: o G.
+            auto alphas = [&](int off, const float4 &a, const float4 &b, f2 &t12, f2 &t22, f2 &r) -> f2 {
+                const float2 t0 = first_row(pxl, pyl[0], a, b);
+                t12 = pack2(t0.x, t0.x + a.w);
+                t22 = pack2(t0.y, t0.y + b.y);
+                const f2 q = fma2(t12, t12, mul2(t22, t22));
+                r = pack2(b.z * ex2_approx(-lo2(q)), b.z * ex2_approx(-hi2(q)));
+                const float al0 = fminf(o.alpha_max, lo2(r)), al1 = fminf(o.alpha_max, hi2(r));
+                return pack2(al0 >= o.alpha_min && off < l0 ? -al0 : 0.f, al1 >= o.alpha_min && off < l1 ? -al1 : 0.f);
+            };
+            auto terms = [&](f2 na, f2 r, const float4 &c2, const float4 &c3, f2 &nw, f2 &dp) {
+                const f2 om = add2(one2, na);  // 1 - alpha >= 1 - alpha_max > 0
+                const f2 iom = pack2(rcp_approx(lo2(om)), rcp_approx(hi2(om)));
+                T2 = mul2(T2, iom);
+                // ed = g . (B - c); dL/dalpha_i = T_i g . (c_i - B_i) + dL/dalpha T_final / (1 - alpha_i)
+                f2 ed = kGeo ? mul2(ngd2, pack2(c3.z, c3.w)) : fma2(ngd2, pack2(c3.z, c3.w), beta2);
+                ed = fma2(ng02, pack2(c2.x, c2.y), fma2(ng12, pack2(c2.z, c2.w), fma2(ng22, pack2(c3.x, c3.y), ed)));
+                if (kGeo) ed = add2(ed, beta2);
+                const f2 ndA = fma2(ed, T2, mul2(ngat2, iom));
+                beta2 = fma2(na, ed, beta2);  // B <- B + alpha (c - B)
+                nw = mul2(na, T2);
+                const f2 d = mul2(ndA, na);
+                // a clamped alpha has zero derivative
+                dp = pack2(lo2(r) <= o.alpha_max ? lo2(d) : 0.f, hi2(r) <= o.alpha_max ? hi2(d) : 0.f);
+            };
+            if constexpr (kGeo) {
+                // one entry after another: the six sums over the lane's two rows, then the warp's
+                for (int i = 0; i < nl; i += kGeoWalk) {
+                    f2 t12[kGeoWalk], t22[kGeoWalk], r[kGeoWalk], na[kGeoWalk];
+                    int off[kGeoWalk];
+#pragma unroll
+                    for (int u = 0; u < kGeoWalk; ++u) {
+                        off[u] = wl[min(i + u, nl - 1)];
+                        const float4 *rc = rec_at(s_rec, off[u]);
+                        na[u] = alphas(off[u], rc[0], rc[1], t12[u], t22[u], r[u]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < kGeoWalk; ++u) {
+                        if (i + u >= nl) break;  // warp-uniform
+                        const float4 *rc = rec_at(s_rec, off[u]);
+                        f2 nw, dp;
+                        terms(na[u], r[u], rc[2], rc[3], nw, dp);
+                        const f2 pt1 = mul2(dp, t12[u]), pt2 = mul2(dp, t22[u]);
+                        float v[NV];
+                        v[0] = lo2(pt1) + hi2(pt1);
+                        v[1] = lo2(pt2) + hi2(pt2);
+                        v[2] = fmaf(hi2(pt1), hi2(t12[u]), lo2(pt1) * lo2(t12[u]));
+                        v[3] = fmaf(hi2(pt1), hi2(t22[u]), lo2(pt1) * lo2(t22[u]));
+                        v[4] = fmaf(hi2(pt2), hi2(t22[u]), lo2(pt2) * lo2(t22[u]));
+                        v[5] = fmaf(hi2(nw), hi2(ngd2), lo2(nw) * lo2(ngd2));
+                        add_sums(__float_as_uint(rc[4].x), v, lo2(na[u]) != 0.f || hi2(na[u]) != 0.f);
+                    }
+                }
+                continue;
+            } else
             for (int g = 0; g < nl; g += kSlots) {
                 const int n = min(kSlots, nl - g);  // warp-uniform
                 // phase 1
 #pragma unroll kBwdUnroll
                 for (int i = 0; i < n; ++i) {
                     const int off = wl[g + i];
-                    const float4 *r = rec_at(s_rec, off);
-                    const float4 a = r[0], b = r[1], c2 = r[2], c3 = r[3];
-                    const float2 t0 = first_row(pxl, pyl[0], a, b);
-                    const f2 t12 = pack2(t0.x, t0.x + a.w), t22 = pack2(t0.y, t0.y + b.y);
-                    const f2 q = fma2(t12, t12, mul2(t22, t22));
-                    const float r0 = b.z * ex2_approx(-lo2(q)), r1 = b.z * ex2_approx(-hi2(q));
-                    const float al0 = fminf(o.alpha_max, r0), al1 = fminf(o.alpha_max, r1);
-                    // negated alphas, zero where the pixel does not blend
-                    const f2 na = pack2(al0 >= o.alpha_min && off < l0 ? -al0 : 0.f,
-                                        al1 >= o.alpha_min && off < l1 ? -al1 : 0.f);
-                    const f2 om = add2(one2, na);  // 1 - alpha >= 1 - alpha_max > 0
-                    const f2 iom = pack2(rcp_approx(lo2(om)), rcp_approx(hi2(om)));
-                    T2 = mul2(T2, iom);
-                    // ed = g . (B - c); dL/dalpha_i = T_i g . (c_i - B_i) + dL/dalpha T_final / (1 - alpha_i)
-                    const f2 ed = fma2(ng02, pack2(c2.x, c2.y),
-                                       fma2(ng12, pack2(c2.z, c2.w),
-                                            fma2(ng22, pack2(c3.x, c3.y), fma2(ngd2, pack2(c3.z, c3.w), beta2))));
-                    const f2 ndA = fma2(ed, T2, mul2(ngat2, iom));
-                    beta2 = fma2(na, ed, beta2);  // B <- B + alpha (c - B)
-                    const f2 nw = mul2(na, T2);
-                    const f2 dp = mul2(ndA, na);
-                    // a clamped alpha has zero derivative
-                    s_term[i * kTermStride + lane] = make_float4(lo2(nw), hi2(nw), r0 <= o.alpha_max ? lo2(dp) : 0.f,
-                                                                 r1 <= o.alpha_max ? hi2(dp) : 0.f);
+                    const float4 *rc = rec_at(s_rec, off);
+                    f2 t12, t22, r, nw, dp;
+                    const f2 na = alphas(off, rc[0], rc[1], t12, t22, r);
+                    terms(na, r, rc[2], rc[3], nw, dp);
+                    s_term[i * kTermStride + lane] = make_float4(lo2(nw), hi2(nw), lo2(dp), hi2(dp));
                 }
                 __syncwarp();
                 // phase 2
@@ -1023,11 +895,9 @@ static size_t list_bytes(int threads, int records) { return sizeof(uint16_t) * (
 static size_t fwd_smem(int threads, int records) {
     return sizeof(float4) * kRecStage * records + list_bytes(threads, records);
 }
-static size_t geo_smem(int threads, int records) {
-    return (sizeof(float4) * 3 + sizeof(uint32_t)) * records + list_bytes(threads, records);
-}
-static size_t bwd_smem(int threads, int records) {
-    return sizeof(float4) * (kRecStage * (size_t)records + (size_t)(threads / 32) * (kSlots * kTermStride + kPixSize)) +
+static size_t bwd_smem(int threads, int records, bool geometric_only) {
+    const size_t per_warp = geometric_only ? 0 : kSlots * kTermStride + kPixSize;
+    return sizeof(float4) * (kRecStage * (size_t)records + (size_t)(threads / 32) * per_warp) +
            list_bytes(threads, records);
 }
 
@@ -1071,8 +941,8 @@ cudaError_t launch_composite_bwd(const RenderWs &ws, const uint32_t *ival, int V
                                  cudaStream_t s) {
     const int B = cam.tile_w * cam.tile_h / kPix;
     const int n_tiles = V * cam.T;
-    const auto kern = geometric_only ? composite_geo_kernel : composite_bwd_kernel;
-    const size_t sm = geometric_only ? geo_smem(B, B * kGeoBatch) : bwd_smem(B, B * kBwdBatch);
+    const auto kern = geometric_only ? composite_bwd_kernel<6> : composite_bwd_kernel<10>;
+    const size_t sm = bwd_smem(B, B * (geometric_only ? kGeoBatch : kBwdBatch), geometric_only);
     // (the kernels' few static words count towards the default limit of 48 KB)
     if (sm > 40 * 1024)
         cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
