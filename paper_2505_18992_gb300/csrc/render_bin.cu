@@ -265,18 +265,31 @@ small_lists_kernel(const uint32_t *__restrict__ by_rank_id, const uint32_t *__re
     for (uint32_t k = lane; k < hits; k += 32u) ival[at + k] = cand[k];
 }
 
-// Emits the (global tile id, record) instances of 256 consecutive depth-ranked
-// Gaussians per block.  The instances of Gaussians spanning at most kCoverRows
-// tile rows are spread evenly over the block's threads; each finds its Gaussian
-// by binary search over the block's local offsets, so a Gaussian covering many
-// tiles does not serialise, and then its tile from the row spans the counting
-// pass stored.  A Gaussian spanning more rows takes one warp: one row per lane,
-// its span from the same row-span function that counted it, a warp prefix of
-// the rows' counts, and each lane writing its row's run of tiles.
+// Emits the (global tile id, record) instances of a chunk of consecutive depth-ranked
+// Gaussians per block.  A Gaussian spanning at most kCoverRows tile rows gives one run
+// of consecutive tiles per row (the spans the counting pass stored), listed in shared
+// memory with its first output position.  The output is then written kEmitWindow
+// positions at a time: each run marks its first position, a running maximum over the
+// marks gives every position its run, and the threads write consecutive positions.  A
+// Gaussian covering many tiles does not serialise.  A Gaussian spanning more rows takes
+// one warp to list its runs: one row per lane, its span from the same row-span function
+// that counted it, and a warp prefix of the rows' counts.
+// Bound: instruction issue and shared memory.  The running maximum costs about 10
+// instructions per instance where a binary search over the Gaussians and a walk over
+// their rows cost 100.  Measured, old -> new: 170k visible pairs, 1.19M instances
+// 28.7 -> 18.9 us; 2.66M pairs, 10.3M 169 -> 141 us; 68k pairs of full-HD views, 1.85M
+// instances 92 -> 30 us (108 us in chunks of 256: kEmitRounds 1, 2, 4: 34, 30, 27 us,
+// and 18.2, 18.9, 26.7 us for the 170k pairs).
 constexpr int kEmitThreads = 256;
+constexpr int kEmitPer = 4;
+#ifndef VPGS_EMIT_ROUNDS
+#define VPGS_EMIT_ROUNDS 2
+#endif
+constexpr int kEmitRounds = VPGS_EMIT_ROUNDS;
+constexpr int kEmitWindow = kEmitThreads * kEmitPer;
+constexpr uint32_t kNoKey = 0xffffffffu;  // the run of a Gaussian whose warp writes its tiles
 
-// 6 blocks per SM (40 registers): the instance loop is latency-bound and wants them
-__global__ void __launch_bounds__(kEmitThreads, 6)
+__global__ void __launch_bounds__(kEmitThreads, 5)
 emit_kernel(const uint32_t *__restrict__ dval, const uint32_t *__restrict__ inst_off,
             const BinRec *__restrict__ bin, const uint32_t *n_vis, const uint32_t *n_inst, int64_t N,
             int64_t M_cap, CamParams cam, uint32_t *__restrict__ ikey, uint32_t *__restrict__ ival,
@@ -297,165 +310,210 @@ emit_kernel(const uint32_t *__restrict__ dval, const uint32_t *__restrict__ inst
     __shared__ uint32_t s_h[4][kRadix];
     const SortPass tps[4] = {p0, p1, p2, p3};
     for (int i = threadIdx.x; i < 4 * kRadix; i += blockDim.x) (&s_h[0][0])[i] = 0u;
-    __shared__ uint32_t s_start[kEmitThreads], s_id[kEmitThreads], s_vb[kEmitThreads];
-    __shared__ uint32_t s_sstart[kEmitThreads];  // starts counting only the small Gaussians' instances
-    __shared__ uint16_t s_large[kEmitThreads];   // chunk positions of the large Gaussians
-    __shared__ uint32_t s_wsum[kEmitThreads / 32][2];
-    __shared__ uint2 s_rect[kEmitThreads];
-    __shared__ float4 s_uv[kEmitThreads];
-    __shared__ Cover s_cv[kEmitThreads];
-    __shared__ uint32_t s_total, s_small, s_nlarge;
+    constexpr int kRuns = kEmitThreads * kCoverRows;
+    __shared__ uint32_t s_first[kRuns], s_key[kRuns];  // runs: first output position, first tile
+    __shared__ uint8_t s_owner[kRuns];                 // the run's Gaussian in the chunk
+    __shared__ __align__(8) uint16_t s_mark[kEmitWindow];
+    __shared__ uint32_t s_start[kEmitThreads], s_id[kEmitThreads];
+    __shared__ uint16_t s_large[kEmitThreads];  // chunk positions of the large Gaussians
+    __shared__ uint16_t s_at[kEmitThreads];     // their first runs
+    __shared__ uint32_t s_warp[kEmitThreads / 32], s_max[kEmitThreads / 32];
+    __shared__ uint32_t s_total, s_nlarge;
     const int64_t nv = *n_vis;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     bool overflow = false;
-    // chunks of kEmitThreads depth-ranked Gaussians, grid-strided (the grid is
-    // sized to what fits on the GPU, not to the capacity)
-    for (int64_t r0 = (int64_t)blockIdx.x * kEmitThreads; r0 < nv && !overflow;
-         r0 += (int64_t)gridDim.x * kEmitThreads) {
-    const int nb = (int)min((int64_t)kEmitThreads, nv - r0);
+    // chunks of consecutive depth-ranked Gaussians, grid-strided (the grid is sized to
+    // what fits on the GPU, not to the capacity): up to kEmitThreads, but fewer where that
+    // would give a block less than kEmitRounds chunks (the nearest Gaussians cover the
+    // most tiles, so few large chunks leave their blocks to finish alone)
+    const int64_t share = (nv / ((int64_t)gridDim.x * kEmitRounds) + 31) & ~int64_t(31);
+    const int chunk = (int)min((int64_t)kEmitThreads, max((int64_t)32, share));
+    for (int64_t r0 = (int64_t)blockIdx.x * chunk; r0 < nv && !overflow; r0 += (int64_t)gridDim.x * chunk) {
+    const int nb = (int)min((int64_t)chunk, nv - r0);
     const uint32_t base = inst_off[r0];
+    uint32_t start = 0u, cnt = 0u, vb = 0u;
+    uint32_t pk[kCoverRows];  // row spans, packed
+    int ty_lo = 0, rows = 0, runs = 0;
+    bool large = false;
+    if (tid == 0) s_nlarge = 0u;
+#pragma unroll
+    for (int r = 0; r < kCoverRows; ++r) pk[r] = kEmptySpan;
     if (tid < nb) {
-        const int64_t r = r0 + tid;
-        const uint32_t id = dval[r];
-        const BinRec br = bin[id];
-        s_start[tid] = inst_off[r] - base;
+        const uint32_t id = dval[r0 + tid];
+        const BinRec &br = bin[id];
+        const uint2 rc = br.rect;
+        const Cover cv = br.cv;
+        cnt = br.cnt;
+        start = inst_off[r0 + tid] - base;
+        s_start[tid] = start;
         s_id[tid] = id;
-        s_rect[tid] = br.rect;
-        s_uv[tid] = br.uv;
-        s_cv[tid] = br.cv;
-        s_vb[tid] = (uint32_t)(id / N) * (uint32_t)cam.T;
+        vb = (uint32_t)(id / N) * (uint32_t)cam.T;
+        ty_lo = (int)(rc.y & 0xffffu);
+        rows = (int)(rc.y >> 16) - ty_lo + 1;
+        large = rows > kCoverRows;
+        if (!large) {
+            const float sp[kCoverRows] = {cv.a.x, cv.a.y, cv.a.z, cv.a.w, cv.b.x, cv.b.y, cv.b.z, cv.b.w};
+#pragma unroll
+            for (int r = 0; r < kCoverRows; ++r)
+                if (r < rows) pk[r] = __float_as_uint(sp[r]);
+        }
         // the block's end offset: the next block's start, or the total
         if (tid == nb - 1) s_total = (r0 + nb < nv ? inst_off[r0 + nb] : *n_inst) - base;
     }
-    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kCoverRows; ++r) runs += (pk[r] & 0xffffu) <= pk[r] >> 16 ? 1 : 0;
+    if (large) runs = rows;
+    uint32_t x, at, n_runs;  // scan of the run counts
+    auto scan_runs = [&]() {
+        x = (uint32_t)runs;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s_warp[warp] = x;
+        __syncthreads();
+        at = x - (uint32_t)runs;
+        n_runs = 0u;
+#pragma unroll
+        for (int w = 0; w < kEmitThreads / 32; ++w) {
+            at += w < warp ? s_warp[w] : 0u;
+            n_runs += s_warp[w];
+        }
+    };
+    scan_runs();
+    const bool listed = n_runs <= (uint32_t)kRuns;  // block-uniform
+    if (!listed) {  // too many rows in the chunk: its large Gaussians write their tiles themselves
+        __syncthreads();
+        if (large) runs = 1;
+        scan_runs();
+    }
     const uint32_t total = s_total;
     if ((int64_t)base + total > M_cap) {
         if (tid == 0) set_status(status, VPGS_ERR_CAPACITY);
         overflow = true;  // block-uniform
         continue;
     }
-    // Gaussians spanning more than kCoverRows tile rows are emitted row-parallel
-    // below; the instance loop covers the others, through a prefix of their counts
-    // (the chunk's own offsets when it has no large Gaussian, the common case)
-    bool large = false;
-    uint32_t cnt = 0u;
-    if (tid < nb) {
-        const uint2 rc = s_rect[tid];
-        large = (int)(rc.y >> 16) - (int)(rc.y & 0xffffu) + 1 > kCoverRows;
-        cnt = (tid + 1 < nb ? s_start[tid + 1] : total) - s_start[tid];
-    }
-    const bool any_large = __syncthreads_or(large) != 0;
-    if (any_large) {
-        uint32_t xs = large ? 0u : cnt, xl = large ? 1u : 0u;  // inclusive scans
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t ys = __shfl_up_sync(0xffffffffu, xs, o), yl = __shfl_up_sync(0xffffffffu, xl, o);
-            if (lane >= o) {
-                xs += ys;
-                xl += yl;
-            }
+    if (large) {
+        if (!listed) {
+            s_first[at] = start;
+            s_key[at] = kNoKey;
+            s_owner[at] = (uint8_t)tid;
         }
-        if (lane == 31) {
-            s_wsum[warp][0] = xs;
-            s_wsum[warp][1] = xl;
-        }
-        __syncthreads();
-        uint32_t ps = 0u, pl = 0u, ts = 0u, tl = 0u;
-#pragma unroll
-        for (int w = 0; w < kEmitThreads / 32; ++w) {
-            if (w < warp) {
-                ps += s_wsum[w][0];
-                pl += s_wsum[w][1];
-            }
-            ts += s_wsum[w][0];
-            tl += s_wsum[w][1];
-        }
-        s_sstart[tid] = ps + xs - (large ? 0u : cnt);
-        if (large) s_large[pl + xl - 1u] = (uint16_t)tid;
-        if (tid == 0) {
-            s_small = ts;
-            s_nlarge = tl;
-        }
-        __syncthreads();
-    }
-    const uint32_t *pref = any_large ? s_sstart : s_start;
-    const uint32_t total_small = any_large ? s_small : total;
-    for (uint32_t e = tid; e < total_small; e += kEmitThreads) {
-        int lo = 0, hi = nb - 1;  // last Gaussian whose (small-instance) start is <= e
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (pref[mid] <= e) lo = mid;
-            else hi = mid - 1;
-        }
-        uint32_t local = e - pref[lo];
-        const uint32_t at = s_start[lo] + local;
-        const uint2 rc = s_rect[lo];
-        const Cover cv = s_cv[lo];
-        const int ty_lo = (int)(rc.y & 0xffffu), ty_hi = (int)(rc.y >> 16);
-        uint32_t key = 0xffffffffu;
-        // spans stored by the counting pass
-        const uint32_t pk[kCoverRows] = {__float_as_uint(cv.a.x), __float_as_uint(cv.a.y),
-                                         __float_as_uint(cv.a.z), __float_as_uint(cv.a.w),
-                                         __float_as_uint(cv.b.x), __float_as_uint(cv.b.y),
-                                         __float_as_uint(cv.b.z), __float_as_uint(cv.b.w)};
+        s_at[tid] = (uint16_t)at;
+        s_large[atomicAdd(&s_nlarge, 1u)] = (uint16_t)tid;
+    } else if (tid < nb) {
+        uint32_t pos = start;
 #pragma unroll
         for (int r = 0; r < kCoverRows; ++r) {
             const uint32_t t0 = pk[r] & 0xffffu, t1 = pk[r] >> 16;
-            const uint32_t n = t0 <= t1 ? t1 - t0 + 1u : 0u;
-            if (key == 0xffffffffu && r <= ty_hi - ty_lo) {
-                if (local < n)
-                    key = s_vb[lo] + (uint32_t)(ty_lo + r) * (uint32_t)cam.tiles_x + t0 + local;
-                else
-                    local -= n;
+            if (t0 <= t1) {
+                s_first[at] = pos;
+                s_key[at] = vb + (uint32_t)(ty_lo + r) * (uint32_t)cam.tiles_x + t0;
+                s_owner[at] = (uint8_t)tid;
+                ++at;
+                pos += t1 - t0 + 1u;
             }
         }
-        if (key == 0xffffffffu) {  // the rows hold fewer tiles than were counted: never in a sound build
-            set_status(status, VPGS_ERR_INTERNAL);
-            key = 0u;
-        }
-        ikey[base + at] = key;
-        ival[base + at] = s_id[lo];
-        add_digits(&s_h[0][0], tps, n_pass, key, dpt);
+        if (pos - start != cnt) set_status(status, VPGS_ERR_INTERNAL);  // never in a sound build
     }
-    // large Gaussians: one warp each, one tile row per lane, a warp prefix of the
-    // rows' counts, each lane writing its row's run of tiles
-    const uint32_t n_large = any_large ? s_nlarge : 0u;
+    // large Gaussians: one warp each, one tile row per lane, a warp prefix of the rows'
+    // counts; each lane lists its row's run (or writes its tiles)
+    __syncthreads();
+    const uint32_t n_large = s_nlarge;
     for (uint32_t j = warp; j < n_large; j += kEmitThreads / 32) {
         const int t = s_large[j];
-        const uint2 rc = s_rect[t];
-        const Cover cv = s_cv[t];
-        const float4 uv = s_uv[t];
+        const uint32_t id = s_id[t];
+        const BinRec &br = bin[id];
+        const uint2 rc = br.rect;
+        const Cover cv = br.cv;
+        const float4 uv = br.uv;
         const int tx_lo = (int)(rc.x & 0xffffu), tx_hi = (int)(rc.x >> 16);
-        const int ty_lo = (int)(rc.y & 0xffffu), ty_hi = (int)(rc.y >> 16);
-        const uint32_t start = s_start[t], end = (t + 1 < nb ? s_start[t + 1] : total);
-        const uint32_t vb = s_vb[t], id = s_id[t];
-        uint32_t running = start;
-        for (int ty0 = ty_lo; ty0 <= ty_hi; ty0 += 32) {  // warp-uniform
+        const int ly_lo = (int)(rc.y & 0xffffu), ly_hi = (int)(rc.y >> 16);
+        const uint32_t begin = s_start[t], end = (t + 1 < nb ? s_start[t + 1] : total);
+        const uint32_t vbase = (uint32_t)(id / N) * (uint32_t)cam.T;
+        uint32_t running = begin;
+        for (int ty0 = ly_lo; ty0 <= ly_hi; ty0 += 32) {  // warp-uniform
             const int ty = ty0 + lane;
             int2 sp = make_int2(1, 0);
-            if (ty <= ty_hi)
+            if (ty <= ly_hi)
                 sp = cover_row(cv, uv.x, uv.z, uv.y, uv.w, ty, tx_lo, tx_hi, cam.tw_shift, cam.tile_h, cam.W, cam.H);
             const uint32_t n = sp.x <= sp.y ? (uint32_t)(sp.y - sp.x + 1) : 0u;
-            uint32_t x = n;
+            uint32_t xs = n;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o) x += y;
+                const uint32_t ys = __shfl_up_sync(0xffffffffu, xs, o);
+                if (lane >= o) xs += ys;
             }
-            const uint32_t at = running + x - n;
-            for (uint32_t k = 0; k < n; ++k) {
-                if (at + k >= end) {  // more tiles than were counted: never in a sound build
+            const uint32_t to = running + xs - n;
+            if (listed && ty <= ly_hi) {
+                const uint32_t k = s_at[t] + (uint32_t)(ty - ly_lo);
+                s_first[k] = n ? to : 0xffffffffu;  // (an empty row starts nowhere)
+                s_key[k] = vbase + (uint32_t)ty * (uint32_t)cam.tiles_x + (uint32_t)sp.x;
+                s_owner[k] = (uint8_t)t;
+            }
+            for (uint32_t k = 0; !listed && k < n; ++k) {
+                if (to + k >= end) {  // more tiles than were counted: never in a sound build
                     set_status(status, VPGS_ERR_INTERNAL);
                     break;
                 }
-                const uint32_t key = vb + (uint32_t)ty * (uint32_t)cam.tiles_x + (uint32_t)sp.x + k;
-                ikey[base + at + k] = key;
-                ival[base + at + k] = id;
+                const uint32_t key = vbase + (uint32_t)ty * (uint32_t)cam.tiles_x + (uint32_t)sp.x + k;
+                ikey[base + to + k] = key;
+                ival[base + to + k] = id;
                 add_digits(&s_h[0][0], tps, n_pass, key, dpt);
             }
-            running += __shfl_sync(0xffffffffu, x, 31);
+            running += __shfl_sync(0xffffffffu, xs, 31);
         }
         if (lane == 0 && running != end) set_status(status, VPGS_ERR_INTERNAL);
+    }
+    uint32_t carry = 0u;  // 1 + the last run that starts before the window
+    for (uint32_t w0 = 0u; w0 < total; w0 += kEmitWindow) {
+        reinterpret_cast<uint2 *>(s_mark)[tid] = make_uint2(0u, 0u);
+        __syncthreads();  // (also the runs' writes before the first window)
+        for (uint32_t k = tid; k < n_runs; k += kEmitThreads) {
+            const uint32_t d = s_first[k] - w0;
+            if (d < (uint32_t)kEmitWindow) s_mark[d] = (uint16_t)(k + 1u);
+        }
+        __syncthreads();
+        // running maximum over the window, four positions per thread
+        const uint2 mk = reinterpret_cast<const uint2 *>(s_mark)[tid];
+        const uint32_t m0 = mk.x & 0xffffu, m1 = max(m0, mk.x >> 16), m2 = max(m1, mk.y & 0xffffu), m3 = max(m2, mk.y >> 16);
+        uint32_t y = m3;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t z = __shfl_up_sync(0xffffffffu, y, o);
+            if (lane >= o) y = max(y, z);
+        }
+        if (lane == 31) s_max[warp] = y;
+        __syncthreads();
+        uint32_t pre = __shfl_up_sync(0xffffffffu, y, 1);
+        if (lane == 0) pre = 0u;
+        pre = max(pre, carry);
+#pragma unroll
+        for (int w = 0; w < kEmitThreads / 32; ++w) {
+            if (w < warp) pre = max(pre, s_max[w]);
+            carry = max(carry, s_max[w]);
+        }
+        reinterpret_cast<uint2 *>(s_mark)[tid] =
+            make_uint2(max(pre, m0) | max(pre, m1) << 16, max(pre, m2) | max(pre, m3) << 16);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kEmitPer; ++j) {
+            const uint32_t d = (uint32_t)(j * kEmitThreads + tid), pos = w0 + d;
+            if (pos < total) {
+                const uint32_t k = s_mark[d] - 1u;
+                uint32_t key = kNoKey;
+                if (k < n_runs) key = s_key[k];
+                else set_status(status, VPGS_ERR_INTERNAL);  // no run before it: never in a sound build
+                if (key != kNoKey) {
+                    key += pos - s_first[k];
+                    ikey[base + pos] = key;
+                    ival[base + pos] = s_id[s_owner[k]];
+                    add_digits(&s_h[0][0], tps, n_pass, key, dpt);
+                }
+            }
+        }
+        __syncthreads();
     }
     __syncthreads();  // the next chunk reuses the shared arrays
     }

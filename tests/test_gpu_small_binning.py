@@ -28,6 +28,8 @@ def _render(arrays, cam, **opts):
     (1, 1, (120, 90), 0.02), (1, 31, (120, 90), 0.02), (1, 33, (120, 90), 0.6), (1, 1024, (120, 90), 0.02),
     (1, 1025, (333, 600), 0.6), (1, 8193, (120, 90), 0.02), (1, 12288, (120, 90), 0.02), (3, 4096, (97, 61), 0.1),
     (3, 2048, (700, 640), 0.3), (1, 6145, (700, 900), 0.02),  # past 15M pairs x tiles: by rank, general
+    # emission: Gaussians of many tile rows, in chunks that hold them as runs and that do not
+    (1, 500, (1900, 1000), 0.5), (1, 300, (400, 4000), 1.5),
     (1, 900, (4120, 20), 0.05), (1, 900, (20, 4120), 0.05)])  # more than 256 columns or rows of tiles
 def test_small_forms_equal_the_general_ones(views, n, size, scale):
     sc = scenes.random_gaussians(n, *size, 1.1 * max(size), seed=n, scale_range=(0.005, scale), n_views=views)
