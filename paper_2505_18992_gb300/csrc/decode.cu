@@ -505,6 +505,57 @@ struct DecGradOut {
     float *features, *offsets, *scaling, *params;
 };
 
+// dst[0..N) += src[0..N) with every load issued before the first store (the compiler must
+// keep a loop of += in order: one load latency per element, 22k cycles for a feature row)
+template <int N>
+VPGS_D void add_row(float *dst, const float *src) {
+    float v[N];
+    if ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
+#pragma unroll
+        for (int k = 0; k < N / 4; ++k) {
+            const float4 q = reinterpret_cast<const float4 *>(dst)[k];
+            v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
+        }
+#pragma unroll
+        for (int k = 0; k < N / 4; ++k)
+            reinterpret_cast<float4 *>(dst)[k] = make_float4(v[4 * k] + src[4 * k], v[4 * k + 1] + src[4 * k + 1],
+                                                             v[4 * k + 2] + src[4 * k + 2], v[4 * k + 3] + src[4 * k + 3]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < N; ++k) v[k] = dst[k];
+#pragma unroll
+        for (int k = 0; k < N; ++k) dst[k] = v[k] + src[k];
+    }
+}
+
+// One anchor's offset gradients of the Gaussians idx[u] (< 0: none; slot first + step u) and
+// their terms of the scaling gradient, loads first.
+template <int N>
+VPGS_D void add_offsets(const DecParams &p, const DecGradIn &gin, const DecGradOut &gout, int64_t a, int first, int step,
+                        const int (&idx)[N], const float (&l)[3], float (&dl)[3]) {
+    float O[N][3], g[N][3], d[N][3];
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        const int64_t at = (a * p.K + first + step * u) * 3;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            g[u][r] = idx[u] >= 0 ? gin.means[3 * (int64_t)idx[u] + r] : 0.f;
+            O[u][r] = idx[u] >= 0 ? p.offsets[at + r] : 0.f;
+            d[u][r] = idx[u] >= 0 && gout.offsets ? gout.offsets[at + r] : 0.f;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        if (idx[u] < 0) continue;
+        const int64_t at = (a * p.K + first + step * u) * 3;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            if (gout.offsets) gout.offsets[at + r] = d[u][r] + g[u][r] * l[r];
+            dl[r] += g[u][r] * O[u][r];
+        }
+    }
+}
+
 constexpr int kBwdAnchors = 64;
 constexpr int kRowIn = 37, kRowH = 33, kRowOut = 73;
 
@@ -559,8 +610,9 @@ decode_bwd_kernel(DecParams p, const double *__restrict__ T, const int32_t *__re
     // which decoded Gaussians of this anchor survived, and where they are
     int idx[kMaxK];
     bool any = false;
-    for (int m = 0; m < K; ++m) {
-        idx[m] = keep ? inv[a * K + m] : -1;
+#pragma unroll
+    for (int m = 0; m < kMaxK; ++m) {
+        idx[m] = keep && m < K ? inv[a * K + m] : -1;
         any |= idx[m] >= 0;
     }
     float l[3] = {0, 0, 0}, dl[3] = {0, 0, 0};
@@ -665,20 +717,14 @@ decode_bwd_kernel(DecParams p, const double *__restrict__ T, const int32_t *__re
         __syncthreads();
     }
     if (!live || !any) return;
-    if (gout.features)
-        for (int k = 0; k < kFeat; ++k) gout.features[kFeat * a + k] += sdi[k];
-    for (int g = 0; g < K; ++g) {
-        const int i = idx[g];
-        if (i < 0) continue;
-        const float *O = p.offsets + (a * K + g) * 3;
-        const float gm[3] = {gin.means[3 * i], gin.means[3 * i + 1], gin.means[3 * i + 2]};
-        for (int r = 0; r < 3; ++r) {
-            if (gout.offsets) gout.offsets[(a * K + g) * 3 + r] += gm[r] * l[r];
-            dl[r] += gm[r] * O[r];
-        }
+    if (gout.features) add_row<kFeat>(gout.features + kFeat * a, sdi);
+    add_offsets(p, gin, gout, a, 0, 1, idx, l, dl);
+    if (gout.scaling) {
+        const float s0 = gout.scaling[3 * a], s1 = gout.scaling[3 * a + 1], s2 = gout.scaling[3 * a + 2];
+        gout.scaling[3 * a] = s0 + dl[0];
+        gout.scaling[3 * a + 1] = s1 + dl[1];
+        gout.scaling[3 * a + 2] = s2 + dl[2];
     }
-    if (gout.scaling)
-        for (int r = 0; r < 3; ++r) gout.scaling[3 * a + r] += dl[r];
 }
 
 // ---------------------------------------------------------------------------
@@ -847,14 +893,40 @@ decode_bwd_mma_kernel(DecParams p, const double *__restrict__ T, const int32_t *
             for (int e = 0; e < 4; ++e) dIn[nt][e] = 0.f;
         __syncthreads();
         const bool keep = s_keep[ta] != 0;
-        int idx[kMaxK];
+        // this thread's Gaussians: slots half, half + 2, ...
+        constexpr int kOwn = kMaxK / 2;
+        int idx[kOwn];
         bool any = false;
-        for (int m = 0; m < K; ++m) {
-            idx[m] = keep ? inv[a * K + m] : -1;
-            any |= idx[m] >= 0;
+#pragma unroll
+        for (int u = 0; u < kOwn; ++u) {
+            const int i0 = keep && 2 * u < K ? inv[a * K + 2 * u] : -1;
+            const int i1 = keep && 2 * u + 1 < K ? inv[a * K + 2 * u + 1] : -1;
+            any |= i0 >= 0 || i1 >= 0;
+            idx[u] = half ? i1 : i0;
         }
 #pragma unroll 1
         for (int j = 0; j < 3; ++j) {
+            // the upstream gradients of this MLP's outputs, in flight during its layers: read
+            // where they were used, they and the row updates below each cost the one warp
+            // per scheduler a load latency (100k street anchors: 175 -> 135 us with both
+            // batched, 240 registers)
+            float up[kOwn][7];
+#pragma unroll
+            for (int u = 0; u < kOwn; ++u) {
+                const int64_t i = idx[u];
+                if (i < 0) continue;
+                if (j == 0) {
+                    up[u][0] = gin.opac[i];
+                } else {
+                    const float *src = j == 1 ? gin.colors : gin.scales;
+#pragma unroll
+                    for (int r = 0; r < 3; ++r) up[u][r] = src[3 * i + r];
+                    if (j == 2) {
+                        const float4 q = reinterpret_cast<const float4 *>(gin.quats)[i];
+                        up[u][3] = q.x; up[u][4] = q.y; up[u][5] = q.z; up[u][6] = q.w;
+                    }
+                }
+            }
             const int ntl2 = j == 0 ? 2 : (j == 1 ? 4 : 9);
             const int kd_steps = out_pad16(j) / 16;
             uint32_t mask = 0u;
@@ -923,13 +995,15 @@ decode_bwd_mma_kernel(DecParams p, const double *__restrict__ T, const int32_t *
                     orw[n] = v;
                     split_bf16(v, S.doT[0][n * kAS + ta], S.doT[1][n * kAS + ta]);
                 };
-                for (int gm = half; gm < K; gm += 2) {
-                    const int i = idx[gm];
+#pragma unroll
+                for (int u = 0; u < kOwn; ++u) {
+                    const int gm = half + 2 * u, i = idx[u];
+                    if (gm >= K) continue;
                     if (j == 0) {
                         float v = 0.f;
                         if (i >= 0) {
                             const float al = tanhf(orw[gm]);
-                            v = gin.opac[i] * (1.f - al * al);
+                            v = up[u][0] * (1.f - al * al);
                         }
                         put(gm, v);
                     } else if (j == 1) {
@@ -941,7 +1015,7 @@ decode_bwd_mma_kernel(DecParams p, const double *__restrict__ T, const int32_t *
                             float v = 0.f;
                             if (i >= 0) {
                                 const float c = sigmoidf_(o[r]);
-                                v = gin.colors[3 * i + r] * c * (1.f - c);
+                                v = up[u][r] * c * (1.f - c);
                             }
                             put(3 * gm + r, v);
                         }
@@ -954,15 +1028,14 @@ decode_bwd_mma_kernel(DecParams p, const double *__restrict__ T, const int32_t *
 #pragma unroll
                             for (int r = 0; r < 3; ++r) {
                                 const float sg = sigmoidf_(o[r]);
-                                const float gs = gin.scales[3 * i + r];
+                                const float gs = up[u][r];
                                 v[r] = gs * l[r] * sg * (1.f - sg);
                                 dl[r] += gs * sg;
                             }
                             const float nrm = sqrtf(o[3] * o[3] + o[4] * o[4] + o[5] * o[5] + o[6] * o[6]);
                             const float inn = 1.0f / nrm;
-                            const float4 gq = reinterpret_cast<const float4 *>(gin.quats)[i];
                             const float qn[4] = {o[3] * inn, o[4] * inn, o[5] * inn, o[6] * inn};
-                            const float gqv[4] = {gq.x, gq.y, gq.z, gq.w};
+                            const float gqv[4] = {up[u][3], up[u][4], up[u][5], up[u][6]};
                             const float dot = qn[0] * gqv[0] + qn[1] * gqv[1] + qn[2] * gqv[2] + qn[3] * gqv[3];
 #pragma unroll
                             for (int r = 0; r < 4; ++r) v[3 + r] = (gqv[r] - qn[r] * dot) * inn;
@@ -1071,19 +1144,11 @@ decode_bwd_mma_kernel(DecParams p, const double *__restrict__ T, const int32_t *
         __syncthreads();
         if (live && any) {
             // the pair splits the features in halves and the Gaussians by parity
-            if (gout.features)
-                for (int k = half * (kFeat / 2); k < (half + 1) * (kFeat / 2); ++k)
-                    gout.features[kFeat * a + k] += S.orow[ta * kOS + k];
-            for (int gm = half; gm < K; gm += 2) {
-                const int i = idx[gm];
-                if (i < 0) continue;
-                const float *O = p.offsets + (a * K + gm) * 3;
-                const float gmn[3] = {gin.means[3 * i], gin.means[3 * i + 1], gin.means[3 * i + 2]};
-                for (int r = 0; r < 3; ++r) {
-                    if (gout.offsets) gout.offsets[(a * K + gm) * 3 + r] += gmn[r] * l[r];
-                    dl[r] += gmn[r] * O[r];
-                }
+            if (gout.features) {
+                constexpr int kHalf = kFeat / 2;
+                add_row<kHalf>(gout.features + kFeat * a + half * kHalf, S.orow + ta * kOS + half * kHalf);
             }
+            add_offsets(p, gin, gout, a, half, 2, idx, l, dl);
         }
         if (half == 1) {
             s_dl[ta][0] = dl[0];
@@ -1091,8 +1156,13 @@ decode_bwd_mma_kernel(DecParams p, const double *__restrict__ T, const int32_t *
             s_dl[ta][2] = dl[2];
         }
         __syncthreads();
-        if (half == 0 && live && any && gout.scaling)
-            for (int r = 0; r < 3; ++r) gout.scaling[3 * a + r] += dl[r] + s_dl[ta][r];
+        if (half == 0 && live && any && gout.scaling) {
+            float v[3];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) v[r] = gout.scaling[3 * a + r];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) gout.scaling[3 * a + r] = v[r] + (dl[r] + s_dl[ta][r]);
+        }
         __syncthreads();  // orow, the staging rows and s_dl are rewritten by the next chunk
     }
     // ---- the block's weight gradients, once
