@@ -745,7 +745,10 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                 beta2 = pack2(ps[0].beta, ps[1].beta);
                 continue;
             }
-            const int l0 = (last[0] - base) * (kRecStage * 16), l1 = (last[1] - base) * (kRecStage * 16);
+            // the offsets the pixels blend below (list positions clamped to the batch: a
+            // position times the record size may not fit 32 bits)
+            const int l0 = min(max(last[0] - base, 0), nb) * (kRecStage * 16),
+                      l1 = min(max(last[1] - base, 0), nb) * (kRecStage * 16);
             // (blend weight, negated; dpow) of the lane's pixels for the record at off, zero
             // where a pixel does not blend; updates T and beta.  t12, t22: the whitened
             // coordinates of the two rows.  na: the negated alphas, masked; r: o G.
