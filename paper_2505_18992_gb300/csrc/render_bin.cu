@@ -182,7 +182,7 @@ small_lists_kernel(const uint32_t *__restrict__ by_rank_id, const uint32_t *__re
                    CamParams cam, uint2 *__restrict__ ranges, uint32_t *__restrict__ ival, uint32_t *cursor,
                    uint32_t *status) {
     grid_dep_enter();
-    if (*status != 0u) return;
+    if (__syncthreads_or(*status != 0u)) return;  // (this launch writes *status: see emit_kernel)
     if ((int64_t)*n_inst > M_cap) {
         if (threadIdx.x == 0) set_status(status, VPGS_ERR_CAPACITY);
         return;
@@ -296,7 +296,15 @@ emit_kernel(const uint32_t *__restrict__ dval, const uint32_t *__restrict__ inst
             uint32_t *status, int n_pass, int dpt, SortPass p0, SortPass p1, SortPass p2, SortPass p3,
             uint32_t *hist, uint32_t *look0) {
     grid_dep_enter();
-    if (*status != 0u) return;  // an earlier kernel failed: dval may hold stale entries
+    // An earlier kernel failed: dval may hold stale entries.  Decided by the block as one:
+    // another block of this launch may write *status meanwhile, and a block whose warps
+    // read it differently would index its runs with words that the absent warps never wrote.
+    if (__syncthreads_or(*status != 0u)) return;
+    // the instance count is final before this launch: every block refuses an overflow alike
+    if ((int64_t)*n_inst > M_cap) {
+        if (threadIdx.x == 0) set_status(status, VPGS_ERR_CAPACITY);
+        return;
+    }
     {
         // the tile sort's first-pass look-back words, for the tiles that will hold
         // instances (the instance count is known from here on)
@@ -390,7 +398,7 @@ emit_kernel(const uint32_t *__restrict__ dval, const uint32_t *__restrict__ inst
     }
     const uint32_t total = s_total;
     if ((int64_t)base + total > M_cap) {
-        if (tid == 0) set_status(status, VPGS_ERR_CAPACITY);
+        if (tid == 0) set_status(status, VPGS_ERR_INTERNAL);  // offsets past their total: never in a sound build
         overflow = true;  // block-uniform
         continue;
     }
