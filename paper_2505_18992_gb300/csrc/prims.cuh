@@ -59,7 +59,9 @@ scan_kernel(Load load, Store store, int64_t n_cap, const uint32_t *n_dev, uint32
             unsigned long long *look, uint32_t *total, uint32_t *status, LookBack lb) {
     constexpr int kTile = kScanThreads * ITEMS;
     grid_dep_enter();
-    if (lb.stop_on_error && *status != 0u) return;
+    // (as a block: another block of this launch may record a timeout meanwhile, and threads
+    // that read the word apart would leave warps to work with what the absent ones never wrote)
+    if (lb.stop_on_error && __syncthreads_or(*status != 0u)) return;
     __shared__ uint32_t s_items[kTile + kTile / 32];
     __shared__ uint32_t s_warp[kScanThreads / kWarp];
     __shared__ uint32_t s_bid, s_excl;
@@ -276,7 +278,7 @@ radix_onesweep_kernel(const uint32_t *__restrict__ key_in, const uint32_t *__res
                       const uint32_t *__restrict__ pass_hist, uint32_t *ticket, uint32_t *look,
                       uint32_t *next_look, uint32_t *status, LookBack lb) {
     grid_dep_enter();
-    if (lb.stop_on_error && *status != 0u) return;
+    if (lb.stop_on_error && __syncthreads_or(*status != 0u)) return;  // (as a block: see scan_kernel)
     constexpr int kWarps = kSortThreads / kWarp;
     constexpr int kSeg = kWarp * ITEMS;  // contiguous items per warp
     constexpr int kTile = kSortThreads * ITEMS;

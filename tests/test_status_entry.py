@@ -36,7 +36,7 @@ def test_the_check_sees_a_split_decision():
     assert _split_decisions(kernel % "__syncthreads_or(*status != 0u)") == []
 
 
-@pytest.mark.parametrize("unit", ["render_bin.cu"])
+@pytest.mark.parametrize("unit", ["render_bin.cu", "prims.cuh"])
 def test_kernels_that_write_the_status_word_enter_as_a_block(unit):
     with open(os.path.join(CSRC, unit)) as f:
         text = f.read()
