@@ -49,7 +49,7 @@ VPGS_D TileCoord tile_coord(int t, const CamParams &cam) {
 
 // Each thread owns kPix pixels of its tile column: rows kPix*ly .. kPix*ly + kPix - 1.
 constexpr int kPix = VPGS_PIX;
-constexpr int kMaxThreads = 512;
+constexpr int kMaxThreads = 512 / kPix;  // tiles hold at most 512 pixels
 #ifndef VPGS_FWD_BATCH
 #define VPGS_FWD_BATCH 2  // records each forward thread stages per batch
 #endif
@@ -113,6 +113,10 @@ VPGS_D bool reaches_box(const float4 &a, const float4 &b, float x0, float x1, fl
 // what they blend.  All 32 lanes take part.  `fine` tells (warp-uniform) whether a
 // listed record is near-degenerate.
 constexpr int kRecStage = 5;  // float4 per staged record: an odd number keeps 16-byte reads by lane conflict-free
+// (the lists are 16-bit: a batch of the largest tile must not hold more records than they reach)
+constexpr bool offsets_fit(int batch) { return (kMaxThreads * batch - 1) * kRecStage * 16 <= 65535; }
+static_assert(offsets_fit(kFwdBatch) && offsets_fit(kBwdBatch) && offsets_fit(kGeoBatch),
+              "the staged batch is larger than the lists' 16-bit offsets reach");
 template <bool kExact, bool kBack>
 VPGS_D int warp_offsets(const float4 *s_rec, int n, float2 band, uint16_t *list, int lane, bool &fine, float xmax,
                         float lg_amin) {
@@ -187,7 +191,7 @@ VPGS_D float2 first_row(float px, float py0, const float4 &a, const float4 &b) {
     return make_float2(fmaf(a.z, dx, a.w * dy), fmaf(b.x, dx, b.y * dy));
 }
 
-// register cap of the forward (0: only the 512-thread launch bound).  96 with 8 entries
+// register cap of the forward (0: only the launch bound of the largest tile).  96 with 8 entries
 // per step: 140 us (room) and 163 us (a street frame whose longest tiles hold 3,600
 // entries: there each warp's own latency counts, not the number of warps); 80 with 6:
 // 144 / 181 us, 72 with 4: 150 / 200 us, 64 with 4: 150 / 230 us.
@@ -547,7 +551,7 @@ constexpr float kOdd = 1e15f;
 
 static_assert(kPix == 2, "the packed forms hold two rows per lane");
 
-// register cap (0: only the 512-thread launch bound).  80: 6 blocks of 4 warps per SM, as
+// register cap (0: only the launch bound of the largest tile).  80: 6 blocks of 4 warps per SM, as
 // many as the shared memory allows; 72: 285 us, 96: 285 us (room; 278 at 80)
 #ifndef VPGS_BWD_MAXREG
 #define VPGS_BWD_MAXREG 80
