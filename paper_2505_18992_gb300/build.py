@@ -37,7 +37,7 @@ def _headers():
 
 
 def _env_flags():
-    """Extra nvcc flags from VPGS_NVCC_FLAGS (e.g. -DVPGS_PIX=2 to retune the compositing geometry)."""
+    """Extra nvcc flags from VPGS_NVCC_FLAGS (e.g. -DVPGS_FWD_MAXREG=80, to retune a kernel)."""
     return os.environ.get("VPGS_NVCC_FLAGS", "").split()
 
 

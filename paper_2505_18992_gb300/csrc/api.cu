@@ -25,9 +25,9 @@ bool valid_opts(const vpgs_render_opts *o) {
     // a warp covers whole rows of a tile: tile_w divides 32
     if (o->tile_w != 4 && o->tile_w != 8 && o->tile_w != 16 && o->tile_w != 32) return false;
     if (o->tile_h < 2 || o->tile_h > 64) return false;
-    // at most 512 pixels per tile; VPGS_PIX adjacent rows per compositing thread, whole warps
+    // at most 512 pixels per tile; kPix adjacent rows per compositing thread, whole warps
     const int B = o->tile_w * o->tile_h;
-    if (o->tile_h % 2 != 0 || B % 64 != 0 || B > 512 || o->tile_h % VPGS_PIX != 0) return false;
+    if (o->tile_h % kPix != 0 || B % 64 != 0 || B > 512) return false;
     if (!(o->alpha_min > 0.f && o->alpha_min < 1.f)) return false;
     if (!(o->alpha_max > o->alpha_min && o->alpha_max < 1.f)) return false;
     if (!(o->t_min > 0.f && o->t_min < 1.f)) return false;

@@ -13,11 +13,13 @@
 #define VPGS_HD __host__ __device__ __forceinline__
 #define VPGS_D __device__ __forceinline__
 
-// Compositing launch geometry (compile-time tuning knobs):
-//   VPGS_PIX    pixels per thread: VPGS_PIX adjacent rows of one column
-#ifndef VPGS_PIX
-#define VPGS_PIX 2
+// A compositing thread owns two adjacent rows of one tile column, which its packed FP32
+// instructions take at once; the kernels have no other form.
+#if defined(VPGS_PIX) && VPGS_PIX != 2
+#error "VPGS_PIX: the compositing kernels hold two rows per thread, no other number"
 #endif
+
+// Launch geometry and arithmetic (compile-time tuning knobs):
 //   VPGS_DEPTH_SORT_GRID, VPGS_OFFSET_SCAN_GRID  blocks per SM of the depth
 //                sort's passes and of the instance-offset scan (0: what is
 //                resident).  Their item count, the visible pairs, is usually far
@@ -39,6 +41,7 @@
 namespace vpgs {
 
 constexpr int kWarp = 32;
+constexpr int kPix = 2;  // pixels per compositing thread
 
 // A launch-geometry value that depends only on the device (an occupancy, a grid
 // size): computed by f() once per device ordinal and kept in `cache` (zero-

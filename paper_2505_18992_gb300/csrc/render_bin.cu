@@ -660,7 +660,7 @@ tile_work_kernel(const int32_t *__restrict__ n_iter, CamParams cam, int n_tiles,
 // forward saves one launch and the backward two, 6 us each by events (320x240: 300
 // tiles of 128 threads).
 bool tiles_ordered(int n_tiles, const CamParams &cam) {
-    const int64_t threads = (int64_t)n_tiles * (cam.tile_w * cam.tile_h / VPGS_PIX);
+    const int64_t threads = (int64_t)n_tiles * (cam.tile_w * cam.tile_h / kPix);
     return VPGS_TILE_ORDER && threads > (int64_t)256 * device_sm_count();
 }
 

@@ -48,7 +48,6 @@ VPGS_D TileCoord tile_coord(int t, const CamParams &cam) {
 }
 
 // Each thread owns kPix pixels of its tile column: rows kPix*ly .. kPix*ly + kPix - 1.
-constexpr int kPix = VPGS_PIX;
 constexpr int kMaxThreads = 512 / kPix;  // tiles hold at most 512 pixels
 #ifndef VPGS_FWD_BATCH
 #define VPGS_FWD_BATCH 2  // records each forward thread stages per batch

@@ -21,6 +21,8 @@ def _compile(unit, flags, out):
     ("render_comp.cu", "-DVPGS_FWD_BATCH=4", "16-bit offsets"),
     ("render_comp.cu", "-DVPGS_BWD_BATCH=4", "16-bit offsets"),
     ("render_comp.cu", "-DVPGS_GEO_BATCH=4", "16-bit offsets"),
+    ("api.cu", "-DVPGS_PIX=1", "two rows per thread"),
+    ("render_comp.cu", "-DVPGS_PIX=4", "two rows per thread"),
 ])
 def test_refused_at_compile_time(unit, flag, reason, tmp_path):
     res = _compile(unit, [flag], tmp_path / "unit.o")
