@@ -766,13 +766,19 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
             };
             auto terms = [&](f2 na, f2 r, const float4 &c2, const float4 &c3, f2 &nw, f2 &dp) {
                 const f2 om = add2(one2, na);  // 1 - alpha >= 1 - alpha_max > 0
+#if VPGS_BWD_RCP
                 const f2 iom = pack2(rcp_approx(lo2(om)), rcp_approx(hi2(om)));
                 T2 = mul2(T2, iom);
+                const f2 gat = mul2(ngat2, iom);
+#else
+                T2 = pack2(lo2(T2) / lo2(om), hi2(T2) / hi2(om));
+                const f2 gat = pack2(lo2(ngat2) / lo2(om), hi2(ngat2) / hi2(om));
+#endif
                 // ed = g . (B - c); dL/dalpha_i = T_i g . (c_i - B_i) + dL/dalpha T_final / (1 - alpha_i)
                 f2 ed = kGeo ? mul2(ngd2, pack2(c3.z, c3.w)) : fma2(ngd2, pack2(c3.z, c3.w), beta2);
                 ed = fma2(ng02, pack2(c2.x, c2.y), fma2(ng12, pack2(c2.z, c2.w), fma2(ng22, pack2(c3.x, c3.y), ed)));
                 if (kGeo) ed = add2(ed, beta2);
-                const f2 ndA = fma2(ed, T2, mul2(ngat2, iom));
+                const f2 ndA = fma2(ed, T2, gat);
                 beta2 = fma2(na, ed, beta2);  // B <- B + alpha (c - B)
                 nw = mul2(na, T2);
                 const f2 d = mul2(ndA, na);
