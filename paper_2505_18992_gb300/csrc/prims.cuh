@@ -495,10 +495,12 @@ inline int64_t sort_blocks(int64_t n, int items) {
 //   ticket [passes] zero;
 //   look   [passes][sort_blocks(n_cap)][256 * sort_dpt(bits)], pass 0's words zero for the tiles
 //          that hold keys (each pass clears the next pass's words of its tiles).
+// ITEMS: keys per thread; NINE: whether `bits` may be 9 (the form of 9-bit digits exists).
+template <int ITEMS, bool NINE>
 inline cudaError_t radix_sort_pairs(const char *name, uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1,
                                     int64_t n_cap, const uint32_t *n_dev, int lo_bit, int bits,
                                     const uint32_t *hist, uint32_t *ticket, uint32_t *look,
-                                    uint32_t *status, cudaStream_t stream, bool *result_in_1, int items,
+                                    uint32_t *status, cudaStream_t stream, bool *result_in_1,
                                     LookBack lb = LookBack{}, int per_sm = 0) {
     SortPass ps[kMaxSortPasses];
     int np = plan_passes(lo_bit, bits, ps);
@@ -506,15 +508,12 @@ inline cudaError_t radix_sort_pairs(const char *name, uint32_t *k0, uint32_t *v0
     if (np == 0 || n_cap == 0) return cudaSuccess;
     if (np > 4) return cudaErrorInvalidValue;
     const int dpt = sort_dpt(bits);
-    const int form = dpt == 2 ? 2 : items == 4 ? 0 : 1;
-    if (items != 4 && items != 16) return cudaErrorInvalidValue;
-    if (dpt == 2 && items != 16) return cudaErrorInvalidValue;
-    const int64_t nb = sort_blocks(n_cap, items);
-    const auto kern = form == 0 ? radix_onesweep_kernel<4, 1>
-                    : form == 1 ? radix_onesweep_kernel<16, 1>
-                                : radix_onesweep_kernel<16, 2>;
-    static std::atomic<int> grids[3][kDeviceCache];  // by form and device
-    const int grid_res = per_device(grids[form], [kern] {
+    static_assert(ITEMS == 4 || ITEMS == 8 || ITEMS == 16 || ITEMS == 32, "keys per thread of a radix pass");
+    if (dpt == 2 && !NINE) return cudaErrorInvalidValue;
+    const int64_t nb = sort_blocks(n_cap, ITEMS);
+    const auto kern = dpt == 2 ? radix_onesweep_kernel<ITEMS, NINE ? 2 : 1> : radix_onesweep_kernel<ITEMS, 1>;
+    static std::atomic<int> grids[2][kDeviceCache];  // per instance, by digit width and device
+    const int grid_res = per_device(grids[dpt - 1], [kern] {
         return resident_grid((const void *)kern, kSortThreads, 0, int64_t(1) << 30);
     });
     const unsigned grid = (unsigned)std::min<int64_t>(grid_cap(grid_res, per_sm), nb);

@@ -755,10 +755,10 @@ cudaError_t build_tile_lists(const GaussIn &g, int V, const CamParams &cam, cons
         // keys per thread: few for a frame's worth of visible Gaussians (short tiles
         // start the look-back chain sooner), more for many views' worth (fewer tiles
         // in the chain); the look-back space is sized for kDepthSortItems, the most tiles
-        const int depth_items = many ? 16 : kDepthSortItems;
-        e = radix_sort_pairs("sort_depth_pass", ws.dkey[0], ws.dval[0], ws.dkey[1], ws.dval[1], L.VN, n_vis,
-                             0, 32, ws.sort_hist[0], ws.counters + CNT_TICKET_D, ws.sort_look[0], ws.status, s,
-                             &in1, depth_items, lb, VPGS_DEPTH_SORT_GRID);
+        const auto depth_sort = many ? radix_sort_pairs<16, false> : radix_sort_pairs<kDepthSortItems, false>;
+        e = depth_sort("sort_depth_pass", ws.dkey[0], ws.dval[0], ws.dkey[1], ws.dval[1], L.VN, n_vis, 0, 32,
+                       ws.sort_hist[0], ws.counters + CNT_TICKET_D, ws.sort_look[0], ws.status, s, &in1, lb,
+                       VPGS_DEPTH_SORT_GRID);
         if (e != cudaSuccess) return e;
         dval = in1 ? ws.dval[1] : ws.dval[0];
         inst_off = in1 ? ws.dkey[0] : ws.dkey[1];  // the depth-sort buffer not holding the result
@@ -783,9 +783,9 @@ cudaError_t build_tile_lists(const GaussIn &g, int V, const CamParams &cam, cons
     if (e != cudaSuccess) return e;
     // 4. stable sort by tile id
     // (digit histograms from the emit kernel)
-    e = radix_sort_pairs("sort_tile_pass", ws.ikey[0], ws.ival[0], ws.ikey[1], ws.ival[1], L.M_cap, n_inst, 0,
-                         L.tile_bits, ws.sort_hist[1], ws.counters + CNT_TICKET_T, ws.sort_look[1],
-                         ws.status, s, &in1, kTileSortItems, lb);
+    e = radix_sort_pairs<kTileSortItems, true>("sort_tile_pass", ws.ikey[0], ws.ival[0], ws.ikey[1], ws.ival[1],
+                                               L.M_cap, n_inst, 0, L.tile_bits, ws.sort_hist[1],
+                                               ws.counters + CNT_TICKET_T, ws.sort_look[1], ws.status, s, &in1, lb);
     if (e != cudaSuccess) return e;
     *sorted_buf = in1 ? 1 : 0;
     if (*sorted_buf != tile_list_buffer(L)) return cudaErrorUnknown;  // never: same pass plan

@@ -23,6 +23,8 @@ def _compile(unit, flags, out):
     ("render_comp.cu", "-DVPGS_GEO_BATCH=4", "16-bit offsets"),
     ("api.cu", "-DVPGS_PIX=1", "two rows per thread"),
     ("render_comp.cu", "-DVPGS_PIX=4", "two rows per thread"),
+    ("render_bin.cu", "-DVPGS_DEPTH_SORT_ITEMS=5", "keys per thread"),
+    ("render_bin.cu", "-DVPGS_TILE_SORT_ITEMS=64", "keys per thread"),
 ])
 def test_refused_at_compile_time(unit, flag, reason, tmp_path):
     res = _compile(unit, [flag], tmp_path / "unit.o")

@@ -95,3 +95,11 @@ def test_ieee_divisions_reach_the_main_walk(case, tmp_path):
             assert_grad_close(got[f"{form}_{k}"], ref["d_" + k], k)
         # T recovered by divisions: other last bits than by reciprocals
         assert any(not np.array_equal(got[f"{form}_{k}"], base[f"{form}_{k}"]) for k in names), form
+
+
+@pytest.mark.parametrize("flags", ["-DVPGS_DEPTH_SORT_ITEMS=8 -DVPGS_TILE_SORT_ITEMS=8",
+                                   "-DVPGS_DEPTH_SORT_ITEMS=16 -DVPGS_TILE_SORT_ITEMS=32"])
+def test_sort_widths_give_the_same_lists(case, tmp_path, flags):
+    got = _variant(case, tmp_path, flags)
+    for k in ("rgb", "depth", "alpha", "t_final", "n_contrib", "n_iter"):
+        assert np.array_equal(got["frame_" + k], case[2]["frame_" + k]), k
