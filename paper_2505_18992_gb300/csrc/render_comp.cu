@@ -68,15 +68,19 @@ constexpr int kGeoBatch = VPGS_GEO_BATCH;
 constexpr int kWalk = VPGS_FWD_WALK;
 
 // Centre and half height of the band of tile-local pixel-centre rows held by
-// this thread's warp.
-VPGS_D float2 warp_rows(const float (&pyl)[kPix]) {
-    float lo = pyl[0], hi = pyl[kPix - 1];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
+// this thread's warp (whole rows of the tile: its width divides 32).
+VPGS_D float2 warp_rows(const CamParams &cam) {
+    const int first = (int)(threadIdx.x & ~31u);
+    const float lo = (float)(kPix * (first >> cam.tw_shift)) + 0.5f;
+    const float hi = (float)(kPix * ((first + 31) >> cam.tw_shift) + kPix - 1) + 0.5f;
     return make_float2(0.5f * (lo + hi), 0.5f * (hi - lo));
+}
+
+// The tile of a block that renders one, loaded beside the status word and not after it:
+// an empty tile costs little but the latency of its few loads, one after another.
+// (Tile blockIdx.x of the order exists for every such block.)
+VPGS_D int first_tile(const uint32_t *order, const uint32_t *work) {
+    return order && !work ? (int)order[blockIdx.x] : (int)blockIdx.x;
 }
 
 // Whether a staged (plain) Gaussian can reach alpha_min at a pixel centre of
@@ -225,13 +229,14 @@ composite_fwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
     const int tid = threadIdx.x, lane = tid & 31;
     uint16_t *wl = reinterpret_cast<uint16_t *>(smem + kRecStage * NT) + (size_t)(tid >> 5) * NT;  // this warp's list
     __shared__ int s_tile;
+    int tile = first_tile(order, work);
     if (*status != 0u) return;
-    const int lx = tid % cam.tile_w, ly = tid / cam.tile_w;
+    const int lx = tid & (cam.tile_w - 1), ly = tid >> cam.tw_shift;
     const float pxl = (float)lx + 0.5f;
     float pyl[kPix];
 #pragma unroll
     for (int q = 0; q < kPix; ++q) pyl[q] = (float)(kPix * ly + q) + 0.5f;
-    const float2 band = warp_rows(pyl);
+    const float2 band = warp_rows(cam);
     const float lg_amin = __log2f(o.alpha_min);
     const f2 one2 = pack2(1.f, 1.f);
     int t = blockIdx.x;
@@ -241,9 +246,9 @@ composite_fwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
             __syncthreads();
             t = s_tile;
             __syncthreads();
+            if (t >= n_tiles) return;
+            tile = order ? (int)order[t] : t;  // launch order -> global tile id
         }
-        if (t >= n_tiles) return;
-        const int tile = order ? (int)order[t] : t;  // launch order -> global tile id
         const TileCoord tc = tile_coord(tile, cam);
         const int px = tc.tx * cam.tile_w + lx;
         const float ox = (float)(tc.tx * cam.tile_w), oy = (float)(tc.ty * cam.tile_h);
@@ -588,12 +593,12 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
     __shared__ int s_max;
     __shared__ int s_odd;
     if (*status != 0u) return;
-    const int lx = tid % cam.tile_w, ly = tid / cam.tile_w;
+    const int lx = tid & (cam.tile_w - 1), ly = tid >> cam.tw_shift;
     const float pxl = (float)lx + 0.5f;
     float pyl[kPix];
 #pragma unroll
     for (int q = 0; q < kPix; ++q) pyl[q] = (float)(kPix * ly + q) + 0.5f;
-    const float2 band = warp_rows(pyl);
+    const float2 band = warp_rows(cam);
     const float lg_amin = __log2f(o.alpha_min);
     const f2 one2 = pack2(1.f, 1.f);
     // adds the lanes' values of one entry to its slots: by a shuffle reduction, or where
@@ -627,11 +632,19 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
         __syncthreads();
         if (t >= n_tiles) return;
         const int tile = order ? (int)order[t] : t;  // launch order -> global tile id
+        const uint2 rg = ranges[tile];
+        // An empty list has no gradients, and its block leaves before the pixels' loads.  They
+        // cost sparse calls 269 us (64 views of 640x480 with ten Gaussians, 76,800 tiles at six
+        // blocks per SM); without them 97 us.  The forward's order load ahead of the status
+        // (first_tile) took it from 187 to 179 us there, of which its images' bytes are 93 us.
+        if (rg.y <= rg.x) {
+            if (!work) return;
+            continue;
+        }
         const TileCoord tc = tile_coord(tile, cam);
         const int px = tc.tx * cam.tile_w + lx;
         const float ox = (float)(tc.tx * cam.tile_w), oy = (float)(tc.ty * cam.tile_h);
         const float xmax = fminf((float)cam.tile_w, (float)cam.W - ox) - 0.5f;  // last pixel centre column
-        const uint2 rg = ranges[tile];
         const int start = (int)rg.x;
         const int64_t HW = (int64_t)cam.H * cam.W;
         // per pixel: T, the negated upstream gradient ng, -dL/dalpha * T_final (ngat) and
