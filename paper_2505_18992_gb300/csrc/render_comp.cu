@@ -519,7 +519,7 @@ VPGS_D bool pair_grad(PixState &p, int jj, const PairEval &e, const float4 &b, c
 // the branching pair code and ten-value shuffle reduction it replaces.  Measured, old ->
 // new: 1M-Gaussian room 1200x680 393 -> 278 us, 8 keyframes of 2M 1848 -> 1369 us, four
 // full-HD views of 34k visible Gaussians 1111 -> 785 us, 10k Gaussians 320x240 41 -> 24 us.
-// kSlots 16 halves the transpose steps but takes 16 KB more per block: 322 us (room).
+// (16 entries halve the transpose steps but take 16 KB more per block: 322 us, room.)
 // The shuffle form remains for the batches that hold a near-degenerate record, and for
 // pixels or records whose magnitudes could turn 0 * x into a NaN (kOdd).
 //
@@ -530,10 +530,7 @@ VPGS_D bool pair_grad(PixState &p, int jj, const PairEval &e, const float4 &b, c
 // in another order, and a tracking run feeds on its own roundings: the signs of the L1
 // loss near its minimum amplify them to pose differences beyond those between two runs.
 // ---------------------------------------------------------------------------
-#ifndef VPGS_BWD_SLOTS
-#define VPGS_BWD_SLOTS 8
-#endif
-constexpr int kSlots = VPGS_BWD_SLOTS;
+constexpr int kSlots = 8;
 #ifndef VPGS_GEO_WALK
 #define VPGS_GEO_WALK 2
 #endif
@@ -546,7 +543,6 @@ constexpr int kDirect = VPGS_BWD_DIRECT;  // at most this many active lanes: per
 #define VPGS_BWD_UNROLL 2
 #endif
 constexpr int kBwdUnroll = VPGS_BWD_UNROLL;
-static_assert(kSlots == 8 || kSlots == 16, "entries per flush");
 constexpr int kTermStride = 33;           // float4 per slot: 32 lanes, padded against bank conflicts
 constexpr int kPixSize = 64 + 32 / kSlots;  // the lanes' gradients: 2 float4 each, one of padding per part of phase 2
 // |upstream gradient| and |colour, depth| from which a pixel or record takes the
@@ -879,30 +875,29 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                         v[9] = fma2(w, pack2(g1.z, g1.w), v[9]);
                     }
                 }
+                // (rs[k] is slot kSlotOf[k]: the lanes that finish an entry then hold slots
+                // 0 1 8 | 2 3 | 4 5 9 | 6 7)
+                constexpr int kSlotOf[NV] = {0, 1, 8, 2, 3, 4, 5, 9, 6, 7};
                 float rs[NV];
 #pragma unroll
-                for (int q = 0; q < NV; ++q) rs[q] = lo2(v[q]) + hi2(v[q]);
-                rs[5] = __fdividef(rs[5], b.z);  // dL/do = sum dpow / o
+                for (int q = 0; q < NV; ++q) rs[q] = lo2(v[kSlotOf[q]]) + hi2(v[kSlotOf[q]]);
+                rs[6] = __fdividef(rs[6], b.z);  // slot 5: dL/do = sum dpow / o
                 // the parts' sums, the values spread over the lanes that held them
                 constexpr int H = (NV + 1) / 2;
+                static_assert(NV == 10 && kSlots == 8, "kSlotOf spreads ten slots over four lanes");
                 half_step<NV, 16>(rs, lane);
-                int lo = (lane & 16) ? H : 0, nq = (lane & 16) ? NV - H : H;
-                if constexpr (kSlots == 8) {
-                    constexpr int Q = (H + 1) / 2;
-                    half_step<H, 8>(rs, lane);
-                    if (lane & 8) {
-                        lo += Q;
-                        nq -= Q;
-                    } else {
-                        nq = min(nq, Q);
-                    }
-                }
+                half_step<H, 8>(rs, lane);
                 if (e < n) {
-                    float *dst = g2d + 10 * (int64_t)__float_as_uint(r[4].x);
-                    constexpr int M = kSlots == 8 ? (H + 1) / 2 : H;
-#pragma unroll
-                    for (int q = 0; q < M; ++q)
-                        if (q < nq && rs[q] != 0.f) atomicAdd(dst + lo + q, rs[q]);
+                    // A Gaussian's row in two instructions, of eight and of two slots: where every
+                    // tile adds to the same few rows, the L2's work per 32-byte sector bounds the
+                    // kernel.  One lane per three consecutive slots took three instructions of
+                    // four scattered words: 500 Gaussians over all of 1920x1080 437 us, now 236
+                    // (by a shuffle reduction per entry 234); room 276 -> 275 us.
+                    const int p = (lane >> 4 & 1) * 2 + (lane >> 3 & 1);
+                    float *row = g2d + 10 * (int64_t)__float_as_uint(r[4].x);
+                    if (rs[0] != 0.f || rs[1] != 0.f)
+                        atomicAdd(reinterpret_cast<float2 *>(row) + p, make_float2(rs[0], rs[1]));
+                    if (!(p & 1) && rs[2] != 0.f) atomicAdd(row + 8 + (p >> 1), rs[2]);
                 }
                 __syncwarp();
             }
