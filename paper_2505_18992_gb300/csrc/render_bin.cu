@@ -286,6 +286,12 @@ constexpr int kEmitPer = 4;
 #define VPGS_EMIT_ROUNDS 2
 #endif
 constexpr int kEmitRounds = VPGS_EMIT_ROUNDS;
+// Fewest Gaussians in a chunk; the grid has a block per as many (up to what is resident).
+// Few large Gaussians need the blocks: with one per 256, 5,000 of half of 1920x1080 each
+// fell to the lane-per-row walk below and took 2550 us, with one per 64 833 us (32: 444,
+// 16: 158).  But 13k and 20k small ones at 320x240 take 8.1 / 5.7 / 6.8 / 8.5 and 7.9 /
+// 7.1 / 9.2 / 10.6 us with a block per 256 / 64 / 32 / 16, so 64: better than 256 for all.
+constexpr int kEmitLeast = 64;
 constexpr int kEmitWindow = kEmitThreads * kEmitPer;
 constexpr uint32_t kNoKey = 0xffffffffu;  // the run of a Gaussian whose warp writes its tiles
 
@@ -334,8 +340,8 @@ emit_kernel(const uint32_t *__restrict__ dval, const uint32_t *__restrict__ inst
     // what fits on the GPU, not to the capacity): up to kEmitThreads, but fewer where that
     // would give a block less than kEmitRounds chunks (the nearest Gaussians cover the
     // most tiles, so few large chunks leave their blocks to finish alone)
-    const int64_t share = (nv / ((int64_t)gridDim.x * kEmitRounds) + 31) & ~int64_t(31);
-    const int chunk = (int)min((int64_t)kEmitThreads, max((int64_t)32, share));
+    const int64_t share = (nv / ((int64_t)gridDim.x * kEmitRounds) + kEmitLeast - 1) & ~int64_t(kEmitLeast - 1);
+    const int chunk = (int)min((int64_t)kEmitThreads, max((int64_t)kEmitLeast, share));
     for (int64_t r0 = (int64_t)blockIdx.x * chunk; r0 < nv && !overflow; r0 += (int64_t)gridDim.x * chunk) {
     const int nb = (int)min((int64_t)chunk, nv - r0);
     const uint32_t base = inst_off[r0];
@@ -774,7 +780,7 @@ cudaError_t build_tile_lists(const GaussIn &g, int V, const CamParams &cam, cons
         return resident_grid((const void *)emit_kernel, kEmitThreads, 0, int64_t(1) << 30);
     });
     VPGS_LAUNCH("emit_instances", s,
-                launch_k(emit_kernel, (unsigned)std::min<int64_t>(std::max<int64_t>((L.VN + kEmitThreads - 1) / kEmitThreads, 1),
+                launch_k(emit_kernel, (unsigned)std::min<int64_t>(std::max<int64_t>((L.VN + kEmitLeast - 1) / kEmitLeast, 1),
                                                           emit_grid),
                               kEmitThreads, 0, s, dval, inst_off, ws.bin, n_vis, n_inst, L.N, L.M_cap,
                                                     cam, ws.ikey[0], ws.ival[0], ws.status, np_tile, sort_dpt(L.tile_bits), tps[0],
