@@ -505,23 +505,27 @@ VPGS_D bool pair_grad(PixState &p, int jj, const PairEval &e, const float4 &b, c
 // (sum dpow / o is the opacity's).  So a warp works in two phases:
 //   1. one lane per column pair of pixels (two rows), as in the forward: walk the
 //      list back to front, update T and beta, and leave (w, dpow) of both pixels in
-//      a slot of shared memory.  Entries that blend into no pixel take no slot.
-//   2. when kSlots entries are collected (or the batch ends): kSlots x (32 / kSlots)
+//      a slot of shared memory.
+//   2. after kSlots entries (or the list's end): kSlots x (32 / kSlots)
 //      lanes, each summing one entry over its share of the warp's pixels in
 //      registers, then log2(32 / kSlots) transpose steps and one global atomic per
 //      (warp, Gaussian, slot).
 // Both phases do their arithmetic on the two rows of a column at once with the
 // packed FP32 instructions (fma.rn.f32x2), which round each half as the scalar
 // ones do.  Lanes that do not blend take part with alpha = 0 (T and beta then keep
-// their values exactly), so a step has no branch but the one on the warp's vote.
+// their values exactly), so a step has no branch.
 // Bound: the shared-memory pipe and latency (issue active 60 %, LSU data pipe 58 %, FMA
 // pipe 42 %; 20 warps per SM).  103 warp instructions per listed entry, against 189 of
 // the branching pair code and ten-value shuffle reduction it replaces.  Measured, old ->
 // new: 1M-Gaussian room 1200x680 393 -> 278 us, 8 keyframes of 2M 1848 -> 1369 us, four
 // full-HD views of 34k visible Gaussians 1111 -> 785 us, 10k Gaussians 320x240 41 -> 24 us.
 // (16 entries halve the transpose steps but take 16 KB more per block: 322 us, room.)
-// The shuffle form remains for the batches that hold a near-degenerate record, and for
-// pixels or records whose magnitudes could turn 0 * x into a NaN (kOdd).
+// The shuffle form remains for near-degenerate records, entry by entry between the
+// others, and for the batches with pixels or records whose magnitudes could turn 0 * x
+// into a NaN (kOdd).  (With whole batches in it for one such record, 1920x1080, old -> so
+// -> entry by entry: 100k flat discs 566 -> 618 -> 456 us, every 20th of 100k a disc
+// 642 -> 494 -> 462, 100k elongated ones 450 -> 491 -> 366, 100k needles, whose long lists
+// blend little, 260 -> 290 -> 312.)
 //
 // The geometric form (NV = 6: no opacity or colour gradient is asked, as in pose
 // tracking) takes phase 1 without branches but sums each entry by shuffles, in the
@@ -713,8 +717,14 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
             bool any_fine;
             const int nl = warp_offsets<true, true>(s_rec, k_end, band, wl, lane, any_fine, xmax, lg_amin);
             const int base = b0 - start;  // list position of the batch's first record
-            if (any_fine || warp_odd || s_odd != 0) {  // warp-uniform
-                // entry by entry, each in its precision form, the warp's sums by shuffles
+            const bool all_slow = warp_odd || s_odd != 0;
+            // one entry in its precision form with branches, the warp's sums by shuffles
+            auto branching = [&](int off) {
+                const float4 *r = rec_at(s_rec, off);
+                const int kk = off / (kRecStage * 16);
+                const uint32_t id = __float_as_uint(r[4].x);
+                const float4 a = r[0], b = r[1], c2 = r[2], c3 = r[3];
+                const float4 c = make_float4(c2.x, c2.z, c3.x, c3.z);
                 PixState ps[kPix];
 #pragma unroll
                 for (int q = 0; q < kPix; ++q) {
@@ -728,33 +738,29 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                     p.gD = -(q ? hi2(ngd2) : lo2(ngd2));
                     p.last = last[q];
                 }
-                for (int i = 0; i < nl; ++i) {
-                    const float4 *r = rec_at(s_rec, wl[i]);
-                    const int kk = wl[i] / (kRecStage * 16);
-                    const uint32_t id = __float_as_uint(r[4].x);
-                    const float4 a = r[0], b = r[1], c2 = r[2], c3 = r[3];
-                    const float4 c = make_float4(c2.x, c2.z, c3.x, c3.z);
-                    float v[NV];
+                float v[NV];
 #pragma unroll
-                    for (int q = 0; q < NV; ++q) v[q] = 0.f;
-                    auto grads = [&](auto fine) -> bool {
-                        constexpr bool kFine = decltype(fine)::value;
-                        float4 f;
-                        if constexpr (kFine) f = fine_extra(rec[id], ox, oy, a.x, a.y);
-                        const float2 t0 = kFine ? make_float2(0.f, 0.f) : first_row(pxl, pyl[0], a, b);
-                        bool any = false;
+                for (int q = 0; q < NV; ++q) v[q] = 0.f;
+                auto grads = [&](auto fine) -> bool {
+                    constexpr bool kFine = decltype(fine)::value;
+                    float4 f;
+                    if constexpr (kFine) f = fine_extra(rec[id], ox, oy, a.x, a.y);
+                    const float2 t0 = kFine ? make_float2(0.f, 0.f) : first_row(pxl, pyl[0], a, b);
+                    bool any = false;
 #pragma unroll
-                        for (int q = 0; q < kPix; ++q) {
-                            const PairEval e = eval_staged<kFine>(q, t0.x, t0.y, pxl, pyl[q], a, b, f, o.alpha_max);
-                            any |= pair_grad(ps[q], base + kk, e, b, c, o, v);
-                        }
-                        return any;
-                    };
-                    const bool act = b.w < 0.f ? grads(std::true_type{}) : grads(std::false_type{});
-                    add_sums(id, v, act);
-                }
+                    for (int q = 0; q < kPix; ++q) {
+                        const PairEval e = eval_staged<kFine>(q, t0.x, t0.y, pxl, pyl[q], a, b, f, o.alpha_max);
+                        any |= pair_grad(ps[q], base + kk, e, b, c, o, v);
+                    }
+                    return any;
+                };
+                const bool act = b.w < 0.f ? grads(std::true_type{}) : grads(std::false_type{});
                 T2 = pack2(ps[0].T, ps[1].T);
                 beta2 = pack2(ps[0].beta, ps[1].beta);
+                add_sums(id, v, act);
+            };
+            if (all_slow || (kGeo && any_fine)) {  // warp-uniform
+                for (int i = 0; i < nl; ++i) branching(wl[i]);
                 continue;
             }
             // the offsets the pixels blend below (list positions clamped to the batch: a
@@ -823,18 +829,34 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                     }
                 }
                 continue;
-            } else
+            } else {
+            auto walk = [&](auto mix) {  // mix: the list holds near-degenerate records
             for (int g = 0; g < nl; g += kSlots) {
                 const int n = min(kSlots, nl - g);  // warp-uniform
                 // phase 1
-#pragma unroll kBwdUnroll
-                for (int i = 0; i < n; ++i) {
+                auto step = [&](int i) {
                     const int off = wl[g + i];
                     const float4 *rc = rec_at(s_rec, off);
                     f2 t12, t22, r, nw, dp;
                     const f2 na = alphas(off, rc[0], rc[1], t12, t22, r);
                     terms(na, r, rc[2], rc[3], nw, dp);
                     s_term[i * kTermStride + lane] = make_float4(lo2(nw), hi2(nw), lo2(dp), hi2(dp));
+                };
+                if constexpr (!decltype(mix)::value) {
+#pragma unroll kBwdUnroll
+                    for (int i = 0; i < n; ++i) step(i);
+                } else {
+                    // near-degenerate entries add their sums at once and leave no terms
+#pragma unroll 1
+                    for (int i = 0; i < n; ++i) {
+                        const int off = wl[g + i];
+                        if (rec_at(s_rec, off)[1].w < 0.f) {
+                            s_term[i * kTermStride + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            branching(off);
+                        } else {
+                            step(i);
+                        }
+                    }
                 }
                 __syncwarp();
                 // phase 2
@@ -900,6 +922,10 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
                     if (!(p & 1) && rs[2] != 0.f) atomicAdd(row + 8 + (p >> 1), rs[2]);
                 }
                 __syncwarp();
+            }
+            };
+            if (any_fine) walk(std::true_type{});
+            else walk(std::false_type{});
             }
         }
         if (!work) return;
