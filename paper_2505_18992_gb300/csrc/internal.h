@@ -40,8 +40,9 @@ int device_sm_count();
 // general emission and sort (kSmallRank).  The small forms cost pairs^2 and pairs x tiles;
 // the lines lie where their measured forward met the general one's with every pair
 // visible (us, small / general): 12,288 pairs x 300 tiles 65 / 75, x 1,200 85 / 94,
-// x 1,900 99 / 96; 12,000 pairs by rank alone 133 / 117; 5,000 pairs x 300 tiles 33 / 65,
-// 1,000 22 / 52.
+// x 1,900 99 / 96; 5,000 pairs x 300 tiles 33 / 65, 1,000 22 / 52.  By rank alone (7,500
+// tiles): 3,000 pairs 88 / 106, 6,000 107 / 121, 8,000 125 / 127, 10,000 142 / 136, 12,000
+// 165 / 144, so the line stays below where they meet.
 enum BinForm { kGeneralBin, kSmallRank, kSmallLists };
 constexpr int64_t kSmallPairs = 12288;       // (below 2^14: a pair fits 16 bits beside its view)
 constexpr int64_t kSmallRankPairs = 6144;

@@ -662,9 +662,12 @@ tile_work_kernel(const int32_t *__restrict__ n_iter, CamParams cam, int n_tiles,
 
 // A launch order pays only where the tiles take more than one round of blocks: with
 // all of them resident at once (256 threads per SM counted, half of what any of the
-// compositing kernels' registers allow) they all start together.  Below the line the
-// forward saves one launch and the backward two, 6 us each by events (320x240: 300
-// tiles of 128 threads).
+// compositing kernels' registers allow) they all start together, and the forward saves
+// one launch and the backward two.  Forward + backward, without / with the order (us, 50k
+// Gaussians of a small scene; 200k of a room): 300 tiles 282 / 291 and 336 / 342, 400
+// tiles 262 / 268 and 323 / 328, 600 tiles 286 / 278 and 303 / 310, 768 tiles 287 / 286 and
+// 312 / 317, 1,200 tiles 297 / 288 and 339 / 312: they meet between 500 and 1,000 tiles by
+// the scene, and the line, 304 tiles of 128 threads, stays where none loses without it.
 bool tiles_ordered(int n_tiles, const CamParams &cam) {
     const int64_t threads = (int64_t)n_tiles * (cam.tile_w * cam.tile_h / kPix);
     return VPGS_TILE_ORDER && threads > (int64_t)256 * device_sm_count();

@@ -530,9 +530,13 @@ VPGS_D bool pair_grad(PixState &p, int jj, const PairEval &e, const float4 &b, c
 // The geometric form (NV = 6: no opacity or colour gradient is asked, as in pose
 // tracking) takes phase 1 without branches but sums each entry by shuffles, in the
 // order and with the roundings it always had: 345 -> 288 us (room), 39 -> 29 us (10k
-// Gaussians at 320x240).  Its two-phase form took 250 us (room), but adds a warp's terms
-// in another order, and a tracking run feeds on its own roundings: the signs of the L1
-// loss near its minimum amplify them to pose differences beyond those between two runs.
+// Gaussians at 320x240).  Where a tile is one warp it gives the branching walk's bits;
+// between warps only the order of the float32 atomics is open, as it was, and a tracking
+// run feeds on its own roundings (the signs of the L1 loss near its minimum).  Ten tracked
+// poses of the small scene differ from a run of the earlier kernel by 1.3e-10 in the median
+// and 8.5e-7 at most, two runs of the earlier kernel by 1.2e-10 and 9.5e-7; of the room by
+// 9.8e-9 and 1.7e-7, and 1.0e-8 and 1.8e-7.  The two-phase form took 250 us (room), but adds
+// a warp's terms in another order: its runs leave that spread twice as often.
 // ---------------------------------------------------------------------------
 constexpr int kSlots = 8;
 #ifndef VPGS_GEO_WALK
@@ -555,8 +559,10 @@ constexpr float kOdd = 1e15f;
 
 static_assert(kPix == 2, "the packed forms hold two rows per lane");
 
-// register cap (0: only the launch bound of the largest tile).  80: 6 blocks of 4 warps per SM, as
-// many as the shared memory allows; 72: 285 us, 96: 285 us (room; 278 at 80)
+// register cap (0: only the launch bound of the largest tile).  80: 6 blocks of 4 warps per
+// SM, as many as the shared memory allows.  Room / 8 keyframes: 72 289 / 1437 us, 80 277 /
+// 1379, 88 288 / 1450, 96 280 / 1412.  The full form spills 52 bytes a thread at 80 (-Xptxas
+// -v; 36 loaded back) and 28 at 96, where one block less is resident.
 #ifndef VPGS_BWD_MAXREG
 #define VPGS_BWD_MAXREG 80
 #endif
@@ -934,9 +940,8 @@ composite_bwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ i
 }
 
 // dynamic shared memory of a compositing block of `threads` threads staging
-// `records` per batch: forward the staged records and the warps' lists; geometric backward s0-s2,
-// the ids and the lists; full backward the staged records, the warps' term slots and
-// pixel gradients, and the lists
+// `records` per batch: the staged records (five float4 each) and the warps' lists; full
+// backward also the warps' term slots and pixel gradients
 static size_t list_bytes(int threads, int records) { return sizeof(uint16_t) * (size_t)(threads / 32) * records; }
 static size_t fwd_smem(int threads, int records) {
     return sizeof(float4) * kRecStage * records + list_bytes(threads, records);
