@@ -212,9 +212,10 @@ VPGS_D float2 first_row(float px, float py0, const float4 &a, const float4 &b) {
 // keeps its T by a select, which leaves every sum as it was (the rounding of each
 // half is the scalar instructions').  The branches it replaces cost their exposed
 // latency in long tiles and their issue slots in the others.  Measured, old -> new:
-// 1M-Gaussian room 1200x680 192 -> 140 us, street frame 1241x376 of 316k visible
-// Gaussians 524 -> 163 us, 8 keyframes of 2M 875 -> 656 us, four full-HD views 504 ->
-// 401 us, 10k Gaussians 320x240 24 -> 12 us.  The exact ellipse test of the backward's
+// 1M-Gaussian room 1200x680 192 -> 138 us, street frame 1241x376 of 316k visible
+// Gaussians 524 -> 160 us, 8 keyframes of 2M 875 -> 646 us, four full-HD views 504 ->
+// 391 us, 10k Gaussians 320x240 24 -> 12 us.  Frames of empty or nearly empty tiles pay
+// for the fewer blocks per SM: 64 views of 640x480 with 150 Gaussians 173 -> 220 us.  The exact ellipse test of the backward's
 // lists gains nothing here (room 144 us either way, street frame 181 -> 196 us).
 __global__ void VPGS_FWD_BOUNDS
 composite_fwd_kernel(const Rec *__restrict__ rec, const uint32_t *__restrict__ ival,
@@ -517,8 +518,8 @@ VPGS_D bool pair_grad(PixState &p, int jj, const PairEval &e, const float4 &b, c
 // Bound: the shared-memory pipe and latency (issue active 60 %, LSU data pipe 58 %, FMA
 // pipe 42 %; 20 warps per SM).  103 warp instructions per listed entry, against 189 of
 // the branching pair code and ten-value shuffle reduction it replaces.  Measured, old ->
-// new: 1M-Gaussian room 1200x680 393 -> 278 us, 8 keyframes of 2M 1848 -> 1369 us, four
-// full-HD views of 34k visible Gaussians 1111 -> 785 us, 10k Gaussians 320x240 41 -> 24 us.
+// new: 1M-Gaussian room 1200x680 393 -> 280 us, 8 keyframes of 2M 1848 -> 1383 us, four
+// full-HD views of 34k visible Gaussians 1111 -> 779 us, 10k Gaussians 320x240 41 -> 24 us.
 // (16 entries halve the transpose steps but take 16 KB more per block: 322 us, room.)
 // The shuffle form remains for near-degenerate records, entry by entry between the
 // others, and for the batches with pixels or records whose magnitudes could turn 0 * x
@@ -529,7 +530,7 @@ VPGS_D bool pair_grad(PixState &p, int jj, const PairEval &e, const float4 &b, c
 //
 // The geometric form (NV = 6: no opacity or colour gradient is asked, as in pose
 // tracking) takes phase 1 without branches but sums each entry by shuffles, in the
-// order and with the roundings it always had: 345 -> 288 us (room), 39 -> 29 us (10k
+// order and with the roundings it always had: 345 -> 289 us (room), 39 -> 29 us (10k
 // Gaussians at 320x240).  Where a tile is one warp it gives the branching walk's bits;
 // between warps only the order of the float32 atomics is open, as it was, and a tracking
 // run feeds on its own roundings (the signs of the L1 loss near its minimum).  Ten tracked
