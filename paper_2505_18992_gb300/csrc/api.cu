@@ -80,7 +80,9 @@ bool make_layout(int64_t N, int V, const vpgs_camera *cam, const vpgs_render_opt
     const int64_t look_a = 4 * sort_blocks(VN1, kDepthSortItems);
     const int64_t look_b = (int64_t)std::max(np_tile, 1) * sort_dpt(L.tile_bits) * sort_blocks(L.M_cap, kTileSortItems);
     L.sort_blocks_max = look_a > look_b ? look_a : look_b;
-    L.off_sort_look = take(4 * kRadix * (size_t)look_a);
+    // (a small call keeps its depth order there instead, a word per pair)
+    const size_t order = bin_form(L) == kGeneralBin ? 0 : 4 * (size_t)VN1;
+    L.off_sort_look = take(std::max(4 * kRadix * (size_t)look_a, order));
     L.off_sort_look_t = take(4 * kRadix * (size_t)look_b);
     // scans: visibility and offsets over V*N items
     L.scan_blocks_max = scan_blocks(VN1);

@@ -735,7 +735,7 @@ cudaError_t build_tile_lists(const GaussIn &g, int V, const CamParams &cam, cons
     if (form != kGeneralBin) {
         // 1-3 at once (the projection left the list and the counts)
         const bool lists = form == kSmallLists;
-        dval = ws.sort_look[0];  // the depth sort's look-back words: at least one per pair
+        dval = ws.sort_look[0];  // the depth sort's look-back words: at least one per pair (make_layout)
         VPGS_LAUNCH("small_rank", s,
                     launch_k(lists ? small_rank_kernel<true> : small_rank_kernel<false>,
                              (unsigned)std::max<int64_t>(std::min<int64_t>((L.VN + kRankOwn - 1) / kRankOwn, 4 * sms), 1),

@@ -2,8 +2,9 @@
 
 Each variant is a copy of the package compiled with VPGS_NVCC_FLAGS and run in a
 process of its own on the same inputs.  One scene is a single tile of 64 pixels, where
-each sum has one order and so one result; the other is large enough for the general
-binning (scans, both radix sorts, emission).
+each sum has one order and so one result; the others are large enough for the general
+binning (scans, both radix sorts, emission) and for the ranking of small calls with the
+general emission and tile sort.
 """
 import os
 import shutil
@@ -22,7 +23,7 @@ pytestmark = pytest.mark.gpu
 
 NAMES = ("means", "scales", "quats", "opacities", "colors")
 
-# run in the variant's process: renders both scenes, one backward of the first
+# run in the variant's process: renders the scenes, two backwards of the first
 CHILD = """
 import sys
 sys.path.insert(0, sys.argv[1])
@@ -32,7 +33,7 @@ build.build()
 from paper_2505_18992_gb300.render import Intrinsics, Renderer
 d = np.load(sys.argv[2])
 res = {}
-for s in ("tile", "frame"):
+for s in ("tile", "frame", "rank"):
     t = lambda k, dt=torch.float32: torch.as_tensor(d[s + "_" + k], dtype=dt, device="cuda")
     W, H, fx, fy, cx, cy = d[s + "_cam"]
     r = Renderer(Intrinsics(int(W), int(H), fx, fy, cx, cy), tile_w=16, tile_h=int(d[s + "_tile_h"]))
@@ -52,10 +53,11 @@ np.savez(sys.argv[3], **res)
 def _inputs():
     tile = scenes.random_gaussians(60, 16, 4, 20.0, 3, scale_range=(0.02, 0.5))
     frame = scenes.random_gaussians(20_000, 320, 240, 300.0, 4, scale_range=(0.005, 0.05))
+    rank = scenes.random_gaussians(6_000, 800, 900, 700.0, 5, scale_range=(0.005, 0.05))
     ref = oracle.render_scene(tile)
     up = masked_upstream(scenes.upstream_grads(5, 1, 4, 16), ref["flags"])
     d = {}
-    for s, sc, h in (("tile", tile, 4), ("frame", frame, 16)):
+    for s, sc, h in (("tile", tile, 4), ("frame", frame, 16), ("rank", rank, 16)):
         c = sc.camera
         d.update({s + "_" + k: a for k, a in zip(NAMES, sc.arrays())})
         d.update({s + "_T": c.T_cw, s + "_tile_h": h, s + "_cam": [c.width, c.height, c.fx, c.fy, c.cx, c.cy]})
@@ -102,4 +104,5 @@ def test_ieee_divisions_reach_the_main_walk(case, tmp_path):
 def test_sort_widths_give_the_same_lists(case, tmp_path, flags):
     got = _variant(case, tmp_path, flags)
     for k in ("rgb", "depth", "alpha", "t_final", "n_contrib", "n_iter"):
-        assert np.array_equal(got["frame_" + k], case[2]["frame_" + k]), k
+        for s in ("frame", "rank"):
+            assert np.array_equal(got[f"{s}_{k}"], case[2][f"{s}_{k}"]), (s, k)
